@@ -201,6 +201,118 @@ cudaError_t launch_field(const DevState& s, int cur, const ParamsOf<S>& p, int w
 }
 
 // ---------------------------------------------------------------------------------
+// Scaled fields of the stored state in FP32 (lbm_net_targets): (u_x, u_y, u_z) * scale and
+// 2 T per node, u and T as node_macro defines them.  One pass over the populations.
+//
+// GB300 issues two FP64 operations per clock and SM, so node_macro's sums and divisions
+// alone take 0.5 ms on 128^3 nodes, 14 times the pass over memory; the single-precision
+// forms therefore carry every sum as an unevaluated pair of floats (Knuth's two-sum, exact
+// error terms) and divide and scale in pairs (Dekker): about 2^-45 relative, far below the
+// rounding of the FP32 result.  lbm_net_targets after 100 steps at 128^3 (FP32, D3Q15):
+// 10.02 -> 7.99 ms with the steps; after 20 steps at 256^3 (FP16): 24.8 -> 9.2 ms (before:
+// four FP64 passes of 0.51 / 3.9 ms each through a staging plane).  Nodes
+// whose pair arithmetic is not finite take node_macro itself.
+// ---------------------------------------------------------------------------------
+struct FloatPair {
+    float hi, lo;
+};
+__device__ __forceinline__ void pair_add(FloatPair& s, float v) {
+    const float t = s.hi + v, b = t - s.hi;
+    s.lo += (s.hi - (t - b)) + (v - b);
+    s.hi = t;
+}
+// a * b of a pair and a pair
+__device__ __forceinline__ FloatPair pair_mul(FloatPair a, FloatPair b) {
+    const float h = a.hi * b.hi;
+    return {h, fmaf(a.hi, b.hi, -h) + fmaf(a.hi, b.lo, a.lo * b.hi)};
+}
+// n / d, inv = the rounded 1 / d.hi
+__device__ __forceinline__ FloatPair pair_div(FloatPair n, FloatPair d, float inv) {
+    const float q = n.hi * inv;
+    const float rem = fmaf(-q, d.hi, n.hi) + fmaf(-q, d.lo, n.lo);
+    return {q, rem * inv};
+}
+
+template <typename S, int Q>
+__global__ void __launch_bounds__(256) targets_kernel(const S* __restrict__ F, const S* __restrict__ G,
+                                                      const float* __restrict__ Tn, ParamsOf<S> p,
+                                                      double scale, float scale_hi, float scale_lo,
+                                                      int aligned, float* __restrict__ out) {
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= p.ncell) return;
+    float v[4];
+    bool done = false;
+    if constexpr (sizeof(typename Storage<S>::real) == 4) {
+        float f[15], g[Q];
+#pragma unroll
+        for (int a = 0; a < 15; ++a) f[a] = Storage<S>::load_f(F[a * p.plane + c], p.wf[a]);
+        float Tref = 0.f;
+        if constexpr (Storage<S>::deviation) Tref = Tn[c];
+#pragma unroll
+        for (int a = 0; a < Q; ++a) g[a] = Storage<S>::load(G[a * p.plane + c], p.wg[a] * Tref);
+        FloatPair r{f[0], 0.f}, t{g[0], 0.f}, j[3] = {{f[1], 0.f}, {f[3], 0.f}, {f[5], 0.f}};
+#pragma unroll
+        for (int a = 1; a < 15; ++a) {
+            pair_add(r, f[a]);
+            if (ex(a) && a != 1) pair_add(j[0], ex(a) > 0 ? f[a] : -f[a]);
+            if (ey(a) && a != 3) pair_add(j[1], ey(a) > 0 ? f[a] : -f[a]);
+            if (ez(a) && a != 5) pair_add(j[2], ez(a) > 0 ? f[a] : -f[a]);
+        }
+#pragma unroll
+        for (int a = 1; a < Q; ++a) pair_add(t, g[a]);
+        pair_add(t, -0.5f * p.heat_source);
+        // minus half the force of this T
+        FloatPair dT = t;
+        pair_add(dT, -p.T0);
+        const FloatPair b = pair_mul(dT, {-0.5f * p.gbeta, 0.f});
+        pair_add(j[0], -0.5f * p.ext_fx);
+        pair_add(j[1], -0.5f * p.ext_fy);
+        pair_add(j[2], -0.5f * p.ext_fz);
+        pair_add(j[2], b.hi);
+        j[2].lo += b.lo;
+        const float inv = 1.0f / r.hi;
+        v[3] = 2.0f * (t.hi + t.lo);
+        done = isfinite(v[3]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const FloatPair u = pair_mul(pair_div(j[d], r, inv), {scale_hi, scale_lo});
+            v[d] = u.hi + u.lo;
+            done = done && isfinite(v[d]);
+        }
+    }
+    if (!done) {
+        double rho, ux, uy, uz, T;
+        node_macro<S, Q>(F, G, Tn, p, c, rho, ux, uy, uz, T);
+        v[0] = (float)(scale * ux);
+        v[1] = (float)(scale * uy);
+        v[2] = (float)(scale * uz);
+        v[3] = (float)(2.0 * T);
+    }
+    if (aligned) {
+        reinterpret_cast<float4*>(out)[c] = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+        for (int d = 0; d < 4; ++d) out[4 * c + d] = v[d];
+    }
+}
+
+template <typename S>
+cudaError_t launch_targets(const DevState& s, int cur, const ParamsOf<S>& p, double scale, float* out,
+                           cudaStream_t st) {
+    const S* F = static_cast<const S*>(s.F[cur]);
+    const S* G = static_cast<const S*>(s.G[cur]);
+    const float* Tn = static_cast<const float*>(s.T[cur]);
+    const unsigned blocks = (unsigned)((p.ncell + 255) / 256);
+    const float hi = (float)scale, lo = (float)(scale - (double)hi);
+    const int aligned = ((uintptr_t)out & 15) == 0;  // a caller's pointer: 16-byte stores where they fit
+    if (s.Q == 15)
+        targets_kernel<S, 15><<<blocks, 256, 0, st>>>(F, G, Tn, p, scale, hi, lo, aligned, out);
+    else
+        targets_kernel<S, 7><<<blocks, 256, 0, st>>>(F, G, Tn, p, scale, hi, lo, aligned, out);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------------
 // Warp / block reductions in FP64.
 // ---------------------------------------------------------------------------------
 __device__ __forceinline__ double warp_sum(double v) {
@@ -466,6 +578,8 @@ cudaError_t launch_nusselt_into(const S* F, const S* G, const ParamsOf<S>& p, do
                                              cudaStream_t);                                        \
     template cudaError_t launch_field<S>(const DevState&, int, const ParamsOf<S>&, int,             \
                                          cudaStream_t);                                            \
+    template cudaError_t launch_targets<S>(const DevState&, int, const ParamsOf<S>&, double,        \
+                                           float*, cudaStream_t);                                  \
     template cudaError_t launch_residual<S>(const DevState&, int, const ParamsOf<S>&, int,          \
                                             cudaStream_t);                                         \
     template cudaError_t launch_nusselt<S>(const DevState&, int, const ParamsOf<S>&, double,        \

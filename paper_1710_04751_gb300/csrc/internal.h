@@ -70,6 +70,10 @@ cudaError_t launch_accumulate_T(float* Tn, const double* src, int64_t n, int fir
 template <typename S>
 cudaError_t launch_field(const DevState& s, int cur, const ParamsOf<S>& p, int which,
                          cudaStream_t st);
+// (u_x, u_y, u_z) * scale and 2 T of every node into out[ncell][4] (device FP32)
+template <typename S>
+cudaError_t launch_targets(const DevState& s, int cur, const ParamsOf<S>& p, double scale, float* out,
+                           cudaStream_t st);
 template <typename S>
 cudaError_t launch_residual(const DevState& s, int cur, const ParamsOf<S>& p, int record,
                             cudaStream_t st);

@@ -9,14 +9,6 @@ using namespace lbm;
 
 namespace {
 
-// out[c * 4 + j] = scale * field[c]
-__global__ void put_channel_kernel(const double* __restrict__ field, int64_t n, int j, double scale,
-                                   float* __restrict__ out) {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-         c += (int64_t)gridDim.x * blockDim.x)
-        out[c * 4 + j] = (float)(scale * field[c]);
-}
-
 // Trilinear resampling of a cell-centred m^3 prediction [voxel][4] onto the nx x ny x nz
 // nodes of a context (node i at (i + 1/2) / nx of the box, clamped at the walls), scaled
 // back to lattice units: u = p * U0, T = p / 2.
@@ -56,17 +48,10 @@ extern "C" int lbm_net_targets(lbm_ctx* c, float* out) {
     if (!c || !out) return fail(c, LBM_EINVAL, "NULL argument%s");
     if (!(c->params.U0 > 0)) return fail(c, LBM_EINVAL, "the context has no velocity scale U0%s");
     DeviceGuard g(c->device);
-    const int64_t n = c->ncell;
-    const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, 65535);
     int rc = with_storage(c->precision, [&](auto tag) {
         using S = decltype(tag);
         const ParamsOf<S> p = dev_params<typename Storage<S>::real>(c);
-        for (int j = 0; j < 4; ++j) {
-            CUDA_OR_FAIL(c, launch_field<S>(c->dev, c->cur, p, j + 1, c->stream));
-            const double scale = j < 3 ? 1.0 / c->params.U0 : 2.0;
-            put_channel_kernel<<<blocks, 256, 0, c->stream>>>(c->dev.staging, n, j, scale, out);
-            CUDA_OR_FAIL(c, cudaGetLastError());
-        }
+        CUDA_OR_FAIL(c, launch_targets<S>(c->dev, c->cur, p, 1.0 / c->params.U0, out, c->stream));
         return LBM_OK;
     });
     if (rc != LBM_OK) return rc;
