@@ -189,7 +189,10 @@ DevParams<real> lbm::dev_params(const lbm_ctx* c) {
 template DevParams<double> lbm::dev_params<double>(const lbm_ctx*);
 template DevParams<float> lbm::dev_params<float>(const lbm_ctx*);
 
-// Wait for all work on a stream, polling an event with a time bound.
+// Wait for all work on a stream, polling an event with a time bound.  The thread polls (and
+// yields) for the first kSpinSeconds: a sleep, however short, returns some 60 us late on
+// Linux, which is as long as a small call runs.  Longer waits sleep between polls.
+static constexpr double kSpinSeconds = 0.02;
 int lbm::wait_stream_for(cudaStream_t stream, double timeout_s, std::string* slot) {
     cudaEvent_t ev;
     cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
@@ -213,7 +216,8 @@ int lbm::wait_stream_for(cudaStream_t stream, double timeout_s, std::string* slo
             cudaEventDestroy(ev);
             return record_error(slot, LBM_ETIMEOUT, "timed out waiting for the GPU%s");
         }
-        std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 5 : 200));
+        if (el < kSpinSeconds) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(100));
     }
     cudaEventDestroy(ev);
     return LBM_OK;

@@ -17,29 +17,36 @@ __device__ int nn_error_word;
 __device__ __align__(128) __nv_bfloat16 nn_probe_operand[128 * 64];
 __device__ __align__(128) float nn_probe_out[128 * 32];
 
-int* error_word() {
-    static int* ptr[64] = {};
+// The device's error word and its mirror in page-locked host memory, into which finish()
+// copies the word behind the stream's work (one pair per device for the process's life).
+struct ErrorWord {
+    int* dev;
+    int* host;
+};
+
+ErrorWord* error_word() {
+    static ErrorWord words[64] = {};
     static std::mutex mu;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
     std::lock_guard<std::mutex> g(mu);
-    if (!ptr[dev]) {
+    if (!words[dev].dev) {
         void* p = nullptr;
+        if (!words[dev].host && cudaMallocHost(&words[dev].host, sizeof(int)) != cudaSuccess) return nullptr;
         if (cudaGetSymbolAddress(&p, nn_error_word) != cudaSuccess) return nullptr;
-        ptr[dev] = static_cast<int*>(p);
+        words[dev].dev = static_cast<int*>(p);
     }
-    return ptr[dev];
+    return &words[dev];
 }
 
 // Waits for the stream and turns a recorded kernel timeout into LBM_ETIMEOUT.
-int finish(cudaStream_t st, int* err) {
+int finish(cudaStream_t st, ErrorWord* err) {
+    if (cudaMemcpyAsync(err->host, err->dev, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        return record_error(nullptr, LBM_ECUDA, "reading the network error word failed%s");
     int rc = wait_stream_for(st, 600.0, nullptr);
     if (rc != LBM_OK) return rc;
-    int h = 0;
-    if (cudaMemcpy(&h, err, sizeof h, cudaMemcpyDeviceToHost) != cudaSuccess)
-        return record_error(nullptr, LBM_ECUDA, "reading the network error word failed%s");
-    if (h != 0) {
-        cudaMemset(err, 0, sizeof(int));
+    if (*static_cast<volatile int*>(err->host) != 0) {
+        cudaMemset(err->dev, 0, sizeof(int));
         return record_error(nullptr, LBM_ETIMEOUT, "a wait inside a tensor-core kernel timed out%s");
     }
     return LBM_OK;
@@ -55,12 +62,12 @@ extern "C" int lbm_nn_gemm_bf16(const void* A, int64_t lda, const void* B, int64
     // the public modes only (the internal split-slice mode writes past C)
     if (out_mode != LBM_GEMM_F32 && out_mode != LBM_GEMM_BF16 && out_mode != LBM_GEMM_F32_ADD)
         return record_error(nullptr, LBM_EINVAL, "invalid GEMM mode%s");
-    int* err = error_word();
+    ErrorWord* err = error_word();
     if (!err) return record_error(nullptr, LBM_ECUDA, "no CUDA device%s");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const cudaError_t e = nn::gemm_bf16(static_cast<const __nv_bfloat16*>(A), lda,
                                         static_cast<const __nv_bfloat16*>(B), ldb, C, ldc, M, N, K,
-                                        out_mode, splits, err, st);
+                                        out_mode, splits, err->dev, st);
     if (e == cudaErrorInvalidValue)
         return record_error(nullptr, LBM_EINVAL, "invalid GEMM shape, stride, alignment or mode%s");
     if (e != cudaSuccess) return record_error(nullptr, LBM_ECUDA, "GEMM launch failed: %s", cudaGetErrorString(e));
@@ -68,7 +75,7 @@ extern "C" int lbm_nn_gemm_bf16(const void* A, int64_t lda, const void* B, int64
 }
 
 extern "C" int lbm_nn_gemm_timeout_probe(void* cuda_stream) {
-    int* err = error_word();
+    ErrorWord* err = error_word();
     if (!err) return record_error(nullptr, LBM_ECUDA, "no CUDA device%s");
     void* op = nullptr;
     void* out = nullptr;
@@ -80,7 +87,7 @@ extern "C" int lbm_nn_gemm_timeout_probe(void* cuda_stream) {
     int rc = finish(st, err);
     if (rc != LBM_OK) return rc;
     const cudaError_t e = nn::gemm_timeout_probe(static_cast<const __nv_bfloat16*>(op),
-                                                 static_cast<float*>(out), err, st);
+                                                 static_cast<float*>(out), err->dev, st);
     if (e != cudaSuccess)
         return record_error(nullptr, LBM_ECUDA, "probe launch failed: %s", cudaGetErrorString(e));
     return finish(st, err);  // LBM_ETIMEOUT when the bounded wait ran out as intended
@@ -94,12 +101,12 @@ extern "C" int lbm_nn_conv3d_wgrad_bf16(const void* X, int batch, int n, int cin
         return record_error(nullptr, LBM_EINVAL,
                             "implicit weight gradient needs n a power of two in 2..256, cin a multiple of 32, "
                             "cout a multiple of 8 in 8..256, Kp >= 27 cin and splits >= 1%s");
-    int* err = error_word();
+    ErrorWord* err = error_word();
     if (!err) return record_error(nullptr, LBM_ECUDA, "no CUDA device%s");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const cudaError_t e = nn::conv_wgrad_implicit(static_cast<const __nv_bfloat16*>(X), batch, n, cin,
                                                   static_cast<const __nv_bfloat16*>(dZ), cout, Kp, ws,
-                                                  (size_t)ws_floats, splits, dWT, 1, err, st);
+                                                  (size_t)ws_floats, splits, dWT, 1, err->dev, st);
     if (e == cudaErrorInvalidValue)
         return record_error(nullptr, LBM_EINVAL, "invalid weight-gradient shape, workspace or alignment%s");
     if (e != cudaSuccess)
@@ -118,12 +125,12 @@ extern "C" int lbm_nn_conv3d_bf16(const void* X, int batch, int n, int cin, cons
         return record_error(nullptr, LBM_EINVAL,
                             "implicit convolution needs cin a multiple of 32, n a power of two in 2..256, "
                             "1 <= cout <= 256 and batch >= 1%s");
-    int* err = error_word();
+    ErrorWord* err = error_word();
     if (!err) return record_error(nullptr, LBM_ECUDA, "no CUDA device%s");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const cudaError_t e = nn::conv_implicit(
         static_cast<const __nv_bfloat16*>(X), batch, n, cin, static_cast<const __nv_bfloat16*>(W), ldw,
-        cout, bias, out, mode == LBM_CONV_BIAS_RELU_BF16 ? nn::CONV_BIAS_RELU_BF16 : nn::CONV_F32, err, st);
+        cout, bias, out, mode == LBM_CONV_BIAS_RELU_BF16 ? nn::CONV_BIAS_RELU_BF16 : nn::CONV_F32, err->dev, st);
     if (e == cudaErrorInvalidValue)
         return record_error(nullptr, LBM_EINVAL, "invalid convolution shape, stride or alignment%s");
     if (e != cudaSuccess)

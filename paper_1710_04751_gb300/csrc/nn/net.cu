@@ -69,6 +69,7 @@ struct lbm_net {
     double* partd;      // per-block partial sums of the loss
     double* loss;
     int* err;
+    double* host;       // page-locked: the loss, then the error word, read behind each call's work
     void* arena;
     size_t arena_bytes;
     int step;
@@ -407,24 +408,19 @@ int update(lbm_net* N) {
     return LBM_OK;
 }
 
-int wait_net(lbm_net* N) {
+// The bounded wait, with the error word (and the loss) copied behind the stream's work into
+// page-locked memory first, so that one wait covers both.
+int wait_net(lbm_net* N, double* loss = nullptr) {
+    int* word = reinterpret_cast<int*>(N->host + 1);
+    NET_CUDA(N, cudaMemcpyAsync(word, N->err, sizeof(int), cudaMemcpyDeviceToHost, N->stream));
+    if (loss) NET_CUDA(N, cudaMemcpyAsync(N->host, N->loss, sizeof(double), cudaMemcpyDeviceToHost, N->stream));
     int rc = wait_stream_for(N->stream, 600.0, &N->msg);
     if (rc != LBM_OK) return rc;
-    int h = 0;
-    NET_CUDA(N, cudaMemcpy(&h, N->err, sizeof h, cudaMemcpyDeviceToHost));
-    if (h) {
+    if (*word) {
         cudaMemset(N->err, 0, sizeof(int));
         return nfail(N, LBM_ETIMEOUT, "a wait inside a tensor-core kernel timed out%s");
     }
-    return LBM_OK;
-}
-
-// The bounded wait (and the kernels' error word) first, then the loss into caller memory:
-// a copy into pageable memory issued before the wait would block without a time limit.
-int finish_with_loss(lbm_net* N, double* loss) {
-    int rc = wait_net(N);
-    if (rc != LBM_OK || !loss) return rc;
-    NET_CUDA(N, cudaMemcpy(loss, N->loss, 8, cudaMemcpyDeviceToHost));
+    if (loss) *loss = N->host[0];
     return LBM_OK;
 }
 
@@ -470,6 +466,7 @@ extern "C" void lbm_net_destroy(lbm_net* N) {
     if (!N) return;
     wait_stream_for(N->stream, 600.0, nullptr);
     if (N->arena) cudaFree(N->arena);
+    if (N->host) cudaFreeHost(N->host);
     delete N;
 }
 
@@ -522,6 +519,7 @@ extern "C" int lbm_net_create(const lbm_net_config* cfg, lbm_net** out) {
     }
     carve(N, static_cast<char*>(N->arena));
     e = cudaMalloc(&N->err, sizeof(int));
+    if (e == cudaSuccess) e = cudaMallocHost(&N->host, 2 * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(N->err, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(N->arena, 0, N->arena_bytes);  // zero moments
     if (e != cudaSuccess) {
@@ -611,7 +609,7 @@ extern "C" int lbm_net_gradients(lbm_net* N, int batch, const float* scalars, co
     NET_RC(upload_scalars(N, batch, scalars));
     NET_RC(forward(N, batch));
     NET_RC(backward(N, batch, targets));
-    return finish_with_loss(N, loss);
+    return wait_net(N, loss);
 }
 
 extern "C" int lbm_net_train_step(lbm_net* N, int batch, const float* scalars, const float* targets,
@@ -621,7 +619,7 @@ extern "C" int lbm_net_train_step(lbm_net* N, int batch, const float* scalars, c
     NET_RC(forward(N, batch));
     NET_RC(backward(N, batch, targets));
     NET_RC(update(N));
-    return finish_with_loss(N, loss);
+    return wait_net(N, loss);
 }
 
 extern "C" int lbm_net_set_lr(lbm_net* N, float lr) {
