@@ -164,32 +164,51 @@ __device__ __forceinline__ UPow<T> upow(T ux, T uy, T uz) {
     return UPow<T>{ux, uy, uz, ux * ux, uy * uy, uz * uz, ux * uy, ux * uz, uy * uz};
 }
 
+// The flow's post-collision central moments (App. A at unit bulk / third / fourth-order
+// rates): first order h = F / 2, shear c_ab and the trace-free parts t_aa = c_aa - rho / 3.
+template <typename T>
+struct FlowRelaxed {
+    T delta, rho;  // rho - 1, rho
+    T hx, hy, hz, cxy, cxz, cyz, txx, tyy, tzz;
+};
+
+// dm: moments of f - w_a up to second order; F: the body force.  Returns u (Eq. 3).
+template <typename T>
+__device__ __forceinline__ FlowRelaxed<T> flow_relax(const Low10<T>& dm, T Fx, T Fy, T Fz, const UnitRates<T>& r,
+                                                     T inv_rho, UPow<T>& u) {
+    FlowRelaxed<T> k;
+    const T h = cst<T>(0.5);
+    k.delta = dm.m0;
+    k.rho = cst<T>(1.0) + k.delta;
+    k.hx = h * Fx, k.hy = h * Fy, k.hz = h * Fz;
+    u = upow<T>((dm.x + k.hx) * inv_rho, (dm.y + k.hy) * inv_rho, (dm.z + k.hz) * inv_rho);
+    // pre-collision second-order central moments about u (the 1/3 of the rest state
+    // cancels in every combination that relaxes): k_ab = m_ab - rho u_a u_b
+    // + (u_a F_b + u_b F_a)/2, k_aa = m_aa - rho u_a^2 + u_a F_a
+    const T kxy = fmad(u.x, k.hy, fmad(u.y, k.hx, dm.xy - k.rho * u.xy));
+    const T kxz = fmad(u.x, k.hz, fmad(u.z, k.hx, dm.xz - k.rho * u.xz));
+    const T kyz = fmad(u.y, k.hz, fmad(u.z, k.hy, dm.yz - k.rho * u.yz));
+    const T sxx = fmad(u.x, Fx, dm.xx - k.rho * u.xx);  // k_xx - 1/3
+    const T syy = fmad(u.y, Fy, dm.yy - k.rho * u.yy);
+    const T szz = fmad(u.z, Fz, dm.zz - k.rho * u.zz);
+    // relaxation: shear at its rates, trace to rho (its equilibrium 3 c_s^2 rho)
+    k.cxy = r.om1[0] * kxy, k.cxz = r.om1[1] * kxz, k.cyz = r.om1[2] * kyz;
+    const T A = r.omA * (sxx - syy);
+    const T B = r.omB * (sxx + syy - cst<T>(2.0) * szz);
+    const T B6 = B * cst<T>(1.0 / 6.0);
+    k.txx = fmad(h, A, B6), k.tyy = B6 - h * A, k.tzz = cst<T>(-2.0) * B6;  // c_aa - rho/3
+    return k;
+}
+
 // Flow (App. A) at unit bulk / third / fourth-order rates.  dm: moments of f - w_a up to
 // second order; F: the body force.  Returns u (Eq. 3) and D, the raw moments of the
 // post-collision f~ - w_a.
 template <typename T>
 __device__ __forceinline__ void flow_unit(const Low10<T>& dm, T Fx, T Fy, T Fz, const UnitRates<T>& r,
                                           T inv_rho, UPow<T>& u, Raw15<T>& D) {
-    const T h = cst<T>(0.5);
-    const T delta = dm.m0;               // rho - 1
-    const T rho = cst<T>(1.0) + delta;
-    const T hx = h * Fx, hy = h * Fy, hz = h * Fz;  // post-collision first central moments
-    u = upow<T>((dm.x + hx) * inv_rho, (dm.y + hy) * inv_rho, (dm.z + hz) * inv_rho);
-    // pre-collision second-order central moments about u (the 1/3 of the rest state
-    // cancels in every combination that relaxes): k_ab = m_ab - rho u_a u_b
-    // + (u_a F_b + u_b F_a)/2, k_aa = m_aa - rho u_a^2 + u_a F_a
-    const T kxy = fmad(u.x, hy, fmad(u.y, hx, dm.xy - rho * u.xy));
-    const T kxz = fmad(u.x, hz, fmad(u.z, hx, dm.xz - rho * u.xz));
-    const T kyz = fmad(u.y, hz, fmad(u.z, hy, dm.yz - rho * u.yz));
-    const T sxx = fmad(u.x, Fx, dm.xx - rho * u.xx);  // k_xx - 1/3
-    const T syy = fmad(u.y, Fy, dm.yy - rho * u.yy);
-    const T szz = fmad(u.z, Fz, dm.zz - rho * u.zz);
-    // relaxation: shear at its rates, trace to rho (its equilibrium 3 c_s^2 rho)
-    const T cxy = r.om1[0] * kxy, cxz = r.om1[1] * kxz, cyz = r.om1[2] * kyz;
-    const T A = r.omA * (sxx - syy);
-    const T B = r.omB * (sxx + syy - cst<T>(2.0) * szz);
-    const T B6 = B * cst<T>(1.0 / 6.0);
-    const T txx = fmad(h, A, B6), tyy = B6 - h * A, tzz = cst<T>(-2.0) * B6;  // c_aa - rho/3
+    const FlowRelaxed<T> k = flow_relax<T>(dm, Fx, Fy, Fz, r, inv_rho, u);
+    const T delta = k.delta, rho = k.rho, hx = k.hx, hy = k.hy, hz = k.hz;
+    const T cxy = k.cxy, cxz = k.cxz, cyz = k.cyz, txx = k.txx, tyy = k.tyy, tzz = k.tzz;
     const T d3 = delta * cst<T>(1.0 / 3.0);
     const T cxx = cst<T>(1.0 / 3.0) * rho + txx, cyy = cst<T>(1.0 / 3.0) * rho + tyy;
     // fourth-order equilibrium E (reading R1), less the rest value 1/9
@@ -269,6 +288,82 @@ __device__ __forceinline__ void thermal7_unit(T phi, T m0, T mx, T my, T mz, con
     d[5] = h * (Dzz + Dz);
     d[6] = h * (Dzz - Dz);
     d[0] = r.halfR - Dxx - Dyy - Dzz;
+}
+
+// ---- u and T imposed after the collision (lbm_init_fields) --------------------------------
+// p <- p~ - p_eq(u, T) + p_eq(v, S): the node keeps its departure from equilibrium and its rho
+// and takes the imposed v and S.  The post-collision state of the collisions above has the u
+// and T they were computed from (the force enters both at the same time level), so p~ -
+// p_eq(u, T) is what is left of D without its equilibrium part, and no population is needed.
+
+// Raw moments of f - w_a: those of f~ - f_eq(rho, u) plus those of f_eq(rho, v) - w_a.
+template <typename T>
+__device__ __forceinline__ void flow_unit_imposed(const Low10<T>& dm, T Fx, T Fy, T Fz, const UnitRates<T>& r,
+                                                  T inv_rho, UPow<T>& u, const UPow<T>& v, Raw15<T>& D) {
+    const FlowRelaxed<T> k = flow_relax<T>(dm, Fx, Fy, Fz, r, inv_rho, u);
+    // fourth-order equilibrium E (reading R1), less f_eq's rho / 9
+    T E9 = cst<T>(0.0);
+    if (r.e4_mode == 0) E9 = fmad(k.txx * k.tyy, inv_rho, cst<T>(1.0 / 3.0) * (k.txx + k.tyy));
+    const T two = cst<T>(2.0), r3 = cst<T>(1.0 / 3.0) * k.rho, d3 = cst<T>(1.0 / 3.0) * k.delta;
+    D.m0 = k.delta;
+    D.x = fmad(k.rho, v.x, k.hx);
+    D.y = fmad(k.rho, v.y, k.hy);
+    D.z = fmad(k.rho, v.z, k.hz);
+    D.xy = fmad(k.rho, v.xy, fmad(u.x, k.hy, fmad(u.y, k.hx, k.cxy)));
+    D.xz = fmad(k.rho, v.xz, fmad(u.x, k.hz, fmad(u.z, k.hx, k.cxz)));
+    D.yz = fmad(k.rho, v.yz, fmad(u.y, k.hz, fmad(u.z, k.hy, k.cyz)));
+    D.xx = fmad(k.rho, v.xx, fmad(u.x, Fx, d3 + k.txx));
+    D.yy = fmad(k.rho, v.yy, fmad(u.y, Fy, d3 + k.tyy));
+    D.zz = fmad(k.rho, v.zz, fmad(u.z, Fz, d3 + k.tzz));
+    const T nxyy = fmad(u.xy, Fy, fmad(u.yy, k.hx, fmad(two * u.y, k.cxy, u.x * k.tyy)));
+    const T nxxy = fmad(u.xy, Fx, fmad(u.xx, k.hy, fmad(two * u.x, k.cxy, u.y * k.txx)));
+    const T nxxz = fmad(u.xz, Fx, fmad(u.xx, k.hz, fmad(two * u.x, k.cxz, u.z * k.txx)));
+    const T nxyz = fmad(u.xy, k.hz, fmad(u.xz, k.hy, fmad(u.yz, k.hx, fmad(u.x, k.cyz, fmad(u.y, k.cxz, u.z * k.cxy)))));
+    const T nxxyy = fmad(u.xy, fmad(u.y, Fx, u.x * Fy), fmad(cst<T>(4.0) * u.xy, k.cxy,
+                         fmad(u.yy, k.txx, fmad(u.xx, k.tyy, E9))));
+    const T rvxy = k.rho * v.xy;
+    D.xyy = fmad(rvxy, v.y, fmad(r3, v.x, nxyy));
+    D.xxy = fmad(rvxy, v.x, fmad(r3, v.y, nxxy));
+    D.xxz = fmad(k.rho * v.xz, v.x, fmad(r3, v.z, nxxz));
+    D.xyz = fmad(rvxy, v.z, nxyz);
+    D.xxyy = fmad(rvxy, v.xy, fmad(r3, v.xx + v.yy, fmad(cst<T>(1.0 / 9.0), k.delta, nxxyy)));
+}
+
+// Raw moments of g - w^phi_a S: thermal15_unit at phi = 0 is g~ - g_eq(phi, u).
+template <typename T>
+__device__ __forceinline__ void thermal15_unit_imposed(T m0, T mx, T my, T mz, const UPow<T>& u,
+                                                       const UnitRates<T>& r, T S, const UPow<T>& v, Raw15<T>& D) {
+    thermal15_unit<T>(cst<T>(0.0), m0, mx, my, mz, u, r, D);
+    const T C2 = r.cs2 * S;
+    D.x = fmad(v.x, S, D.x);
+    D.y = fmad(v.y, S, D.y);
+    D.z = fmad(v.z, S, D.z);
+    D.xy = fmad(v.xy, S, D.xy);
+    D.xz = fmad(v.xz, S, D.xz);
+    D.yz = fmad(v.yz, S, D.yz);
+    D.xx = fmad(v.xx, S, D.xx);
+    D.yy = fmad(v.yy, S, D.yy);
+    D.zz = fmad(v.zz, S, D.zz);
+    D.xyy = fmad(v.xy * v.y, S, fmad(v.x, C2, D.xyy));
+    D.xxy = fmad(v.xy * v.x, S, fmad(v.y, C2, D.xxy));
+    D.xxz = fmad(v.xz * v.x, S, fmad(v.z, C2, D.xxz));
+    D.xyz = fmad(v.xy * v.z, S, D.xyz);
+    D.xxyy = fmad(v.xx * v.yy, S, fmad(v.xx + v.yy, C2, D.xxyy));
+}
+
+template <typename T>
+__device__ __forceinline__ void thermal7_unit_imposed(T m0, T mx, T my, T mz, const UPow<T>& u,
+                                                      const UnitRates<T>& r, T S, const UPow<T>& v, T (&d)[7]) {
+    thermal7_unit<T>(cst<T>(0.0), m0, mx, my, mz, u, r, d);
+    const T h = cst<T>(0.5);
+    const T Dx = v.x * S, Dy = v.y * S, Dz = v.z * S, Dxx = v.xx * S, Dyy = v.yy * S, Dzz = v.zz * S;
+    d[1] += h * (Dxx + Dx);
+    d[2] += h * (Dxx - Dx);
+    d[3] += h * (Dyy + Dy);
+    d[4] += h * (Dyy - Dy);
+    d[5] += h * (Dzz + Dz);
+    d[6] += h * (Dzz - Dz);
+    d[0] -= Dxx + Dyy + Dzz;
 }
 
 // Whether a context's rates are the paper's unit higher-order rates (host side).

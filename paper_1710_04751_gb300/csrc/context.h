@@ -56,6 +56,9 @@ struct lbm_ctx {
     cudaStream_t capture = nullptr;
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
     bool graphs_failed = false;  // capture not possible here: launch the steps one by one
+    // (u_x, u_y, u_z, T) of lbm_init_fields in the arithmetic type, for its rounds of one step
+    // and a reimposition; allocated at the first such call, freed with the context
+    void* imposed = nullptr;
     int64_t cell0 = 0;  // global index of cell 0 (slabs of a larger grid), for the initial noise
 };
 
@@ -95,6 +98,10 @@ int create_context(const lbm_grid* grid, int lattice, const lbm_params* params,
 int transfer_cells(lbm_ctx* c, double* f, double* g, const double* fin, const double* gin,
                    int64_t first, int64_t count, int64_t hstride);
 int transfer_done(lbm_ctx* c, bool uploaded);
+
+// Whether lbm_init_fields runs each of its rounds as one kernel on this context (and reads the
+// given fields only before the first); makes room for the packed fields at the first call.
+bool rounds_fused(lbm_ctx* c);
 
 // lbm_fields for cells [first, first + count): outs[w] (rho, ux, uy, uz, T; NULL = skip)
 // receive count values each.

@@ -152,6 +152,30 @@ cudaError_t launch_reimpose(const DevState& s, int cur, const ParamsOf<S>& p, co
     return cudaGetLastError();
 }
 
+// FP64 fields -> quadruples (u_x, u_y, u_z, T) of the arithmetic type.
+template <typename real>
+__global__ void pack_imposed_kernel(const double* __restrict__ ux, const double* __restrict__ uy,
+                                    const double* __restrict__ uz, const double* __restrict__ T, int64_t n,
+                                    real* __restrict__ out) {
+    const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= n) return;
+    struct alignas(4 * sizeof(real)) Four {
+        real x, y, z, t;
+    };
+    reinterpret_cast<Four*>(out)[c] = {(real)ux[c], (real)uy[c], (real)uz[c], (real)T[c]};
+}
+
+template <typename real>
+cudaError_t launch_pack_imposed(const double* ux, const double* uy, const double* uz, const double* T,
+                                int64_t n, real* out, cudaStream_t st) {
+    pack_imposed_kernel<real><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(ux, uy, uz, T, n, out);
+    return cudaGetLastError();
+}
+template cudaError_t launch_pack_imposed<double>(const double*, const double*, const double*, const double*,
+                                                 int64_t, double*, cudaStream_t);
+template cudaError_t launch_pack_imposed<float>(const double*, const double*, const double*, const double*,
+                                                int64_t, float*, cudaStream_t);
+
 template <typename S>
 cudaError_t launch_set_fields(const DevState& s, int cur, const ParamsOf<S>& p, const double* rho,
                               const double* ux, const double* uy, const double* uz,

@@ -1,6 +1,8 @@
 // bridge.cu -- between the solver and the warm-start network: the training targets of a
 // solved cavity, and a cavity started from the network's prediction (the equilibria of
 // the predicted fields, lbm_set_fields), resampled trilinearly when the grids differ.
+#include <algorithm>
+
 #include "../context.h"
 #include "lbm_net.h"
 #include "nn.h"
@@ -12,34 +14,91 @@ namespace {
 // Trilinear resampling of a cell-centred m^3 prediction [voxel][4] onto the nx x ny x nz
 // nodes of a context (node i at (i + 1/2) / nx of the box, clamped at the walls), scaled
 // back to lattice units: u = p * U0, T = p / 2.
-__global__ void resample_kernel(const float* __restrict__ pred, int m, int nx, int ny, int nz,
-                                double U0, double* __restrict__ ux, double* __restrict__ uy,
-                                double* __restrict__ uz, double* __restrict__ T) {
-    const int64_t total = (int64_t)nx * ny * nz;
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < total;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        const int i = (int)(c % nx), j = (int)((c / nx) % ny), k = (int)(c / ((int64_t)nx * ny));
-        const double s[3] = {(i + 0.5) * m / nx - 0.5, (j + 0.5) * m / ny - 0.5, (k + 0.5) * m / nz - 0.5};
-        int lo[3];
-        double w[3];
-        for (int d = 0; d < 3; ++d) {
-            const double v = fmin(fmax(s[d], 0.0), (double)(m - 1));
-            lo[d] = min((int)floor(v), m - 2 < 0 ? 0 : m - 2);
-            w[d] = m == 1 ? 0.0 : v - lo[d];
+//
+// FP64 arithmetic, of which GB300 issues two operations per clock and SM: the eight-corner sum
+// per node took 0.57 ms at 64^3 -> 128^3 (three divisions, 32 conversions and 32 products a
+// node).  A block therefore takes whole x-rows: the row of the prediction at the node row's
+// (y, z) is interpolated once into shared memory (4 m values), and every node adds one
+// interpolation in x with weights its thread keeps from row to row: about 30 operations a node
+// instead of 170.  A warm start 64^3 -> 128^3 with 50 rounds and the fields read back, with
+// the fused rounds (launch_step_imposed): 15.6 -> 4.6 ms.
+constexpr int kResampleThreads = 128, kResampleRows = 16;
+
+// Position of node i of n on an axis of m cells: cells lo and hi = lo + 1 with weights 1 - w
+// and w.  A cell of weight 0 must not enter the sum (its value may not be finite): `one` is 1
+// when only lo counts, 2 when only hi does.
+struct AxisCell {
+    double w, v;  // v = 1 - w
+    int lo, hi, one;
+};
+__device__ __forceinline__ AxisCell axis_cell(int i, int n, int m) {
+    const double s = (i + 0.5) * m / n - 0.5;
+    const double p = fmin(fmax(s, 0.0), (double)(m - 1));
+    AxisCell a;
+    a.lo = min((int)floor(p), m - 2 < 0 ? 0 : m - 2);
+    a.hi = min(a.lo + 1, m - 1);
+    a.w = m == 1 ? 0.0 : p - a.lo;
+    a.v = 1.0 - a.w;
+    a.one = a.w == 0.0 ? 1 : a.v == 0.0 ? 2 : 0;
+    return a;
+}
+__device__ __forceinline__ double mix(double l, double h, const AxisCell& a) {
+    const double r = fma(a.w, h, a.v * l);
+    return a.one == 0 ? r : a.one == 1 ? l : h;
+}
+
+__global__ void __launch_bounds__(kResampleThreads)
+    resample_kernel(const float* __restrict__ pred, int m, int nx, int ny, int nz, double U0,
+                    double* __restrict__ ux, double* __restrict__ uy, double* __restrict__ uz,
+                    double* __restrict__ T) {
+    extern __shared__ double row[];  // [4][m]
+    __shared__ AxisCell cell[2][kResampleRows];
+    const int i = blockIdx.x * kResampleThreads + threadIdx.x;
+    const AxisCell x = axis_cell(i < nx ? i : 0, nx, m);
+    const int64_t rows = (int64_t)ny * nz;
+    for (int64_t r0 = (int64_t)blockIdx.y * kResampleRows; r0 < rows; r0 += (int64_t)gridDim.y * kResampleRows) {
+        __syncthreads();  // the cells before are read
+        if (threadIdx.x < 2 * kResampleRows) {
+            const int64_t r = min(r0 + threadIdx.x % kResampleRows, rows - 1);
+            const int k = (int)(r / ny), j = (int)(r - (int64_t)k * ny);
+            if (threadIdx.x < kResampleRows) cell[0][threadIdx.x] = axis_cell(j, ny, m);
+            else cell[1][threadIdx.x - kResampleRows] = axis_cell(k, nz, m);
         }
-        double acc[4] = {0, 0, 0, 0};
-        for (int corner = 0; corner < 8; ++corner) {
-            const int dx = corner & 1, dy = (corner >> 1) & 1, dz = corner >> 2;
-            const double wt = (dx ? w[0] : 1 - w[0]) * (dy ? w[1] : 1 - w[1]) * (dz ? w[2] : 1 - w[2]);
-            if (wt == 0.0) continue;
-            const int64_t v = ((int64_t)(lo[2] + dz) * m + (lo[1] + dy)) * m + (lo[0] + dx);
-            for (int q = 0; q < 4; ++q) acc[q] += wt * pred[v * 4 + q];
+        for (int q = 0; q < kResampleRows && r0 + q < rows; ++q) {
+            __syncthreads();  // the cells are there, the row before is read
+            const AxisCell y = cell[0][q], z = cell[1][q];
+            const float* p00 = pred + ((int64_t)z.lo * m + y.lo) * m * 4;
+            const float* p01 = pred + ((int64_t)z.lo * m + y.hi) * m * 4;
+            const float* p10 = pred + ((int64_t)z.hi * m + y.lo) * m * 4;
+            const float* p11 = pred + ((int64_t)z.hi * m + y.hi) * m * 4;
+            for (int e = threadIdx.x; e < 4 * m; e += kResampleThreads)
+                row[(e & 3) * m + (e >> 2)] =
+                    ((e & 3) == 3 ? 0.5 : U0) * mix(mix(p00[e], p01[e], y), mix(p10[e], p11[e], y), z);
+            __syncthreads();
+            if (i < nx) {
+                const int64_t c = (r0 + q) * nx + i;
+                ux[c] = mix(row[x.lo], row[x.hi], x);
+                uy[c] = mix(row[m + x.lo], row[m + x.hi], x);
+                uz[c] = mix(row[2 * m + x.lo], row[2 * m + x.hi], x);
+                T[c] = mix(row[3 * m + x.lo], row[3 * m + x.hi], x);
+            }
         }
-        ux[c] = acc[0] * U0;
-        uy[c] = acc[1] * U0;
-        uz[c] = acc[2] * U0;
-        T[c] = 0.5 * acc[3];
     }
+}
+
+cudaError_t launch_resample(const float* pred, int m, const lbm_grid& g, double U0, double* out, int64_t n,
+                            cudaStream_t st) {
+    const size_t smem = (size_t)4 * m * sizeof(double);
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(resample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)std::min<size_t>(smem, 220 * 1024));
+        if (e != cudaSuccess) return e;
+    }
+    const int64_t chunks = ((int64_t)g.ny * g.nz + kResampleRows - 1) / kResampleRows;
+    const dim3 grid((g.nx + kResampleThreads - 1) / kResampleThreads, (unsigned)std::min<int64_t>(chunks, 65535));
+    resample_kernel<<<grid, kResampleThreads, smem, st>>>(pred, m, g.nx, g.ny, g.nz, U0, out, out + n,
+                                                          out + 2 * n, out + 3 * n);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -64,16 +123,20 @@ extern "C" int lbm_net_warm_start(lbm_ctx* c, const float* pred, int m, int iter
     if (!(c->params.U0 > 0)) return fail(c, LBM_EINVAL, "the context has no velocity scale U0%s");
     DeviceGuard g(c->device);
     const int64_t n = c->ncell;
-    double* buf = nullptr;
-    cudaError_t e = cudaMalloc(&buf, (size_t)4 * n * sizeof(double));
-    if (e != cudaSuccess) return fail(c, LBM_ENOMEM, "cudaMalloc failed: %s", cudaGetErrorString(e));
-    const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, 65535);
-    resample_kernel<<<blocks, 256, 0, c->stream>>>(pred, m, c->grid.nx, c->grid.ny, c->grid.nz,
-                                                   c->params.U0, buf, buf + n, buf + 2 * n, buf + 3 * n);
-    e = cudaGetLastError();
+    // The FP64 fields go to the flow planes of the buffer the next step writes when nothing
+    // reads them after lbm_init_fields has (FP32 and FP64); else to memory of their own.
+    const bool dev16 = c->precision == LBM_FP16_DEV || c->precision == LBM_BF16_DEV;
+    const bool lend = !dev16 && (iterations == 0 || rounds_fused(c));
+    double* own = nullptr;
+    if (!lend) {
+        const cudaError_t e = cudaMalloc(&own, (size_t)4 * n * sizeof(double));
+        if (e != cudaSuccess) return fail(c, LBM_ENOMEM, "cudaMalloc failed: %s", cudaGetErrorString(e));
+    }
+    double* buf = lend ? static_cast<double*>(c->dev.F[c->cur ^ 1]) : own;
+    const cudaError_t e = launch_resample(pred, m, c->grid, c->params.U0, buf, n, c->stream);
     int rc = e == cudaSuccess
                  ? lbm_init_fields(c, nullptr, buf, buf + n, buf + 2 * n, buf + 3 * n, iterations)
                  : fail(c, LBM_ECUDA, "resampling failed: %s", cudaGetErrorString(e));
-    cudaFree(buf);  // lbm_init_fields waited for the stream
+    if (own) cudaFree(own);  // lbm_init_fields waited for the stream
     return rc;
 }

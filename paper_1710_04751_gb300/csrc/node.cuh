@@ -103,12 +103,15 @@ __device__ __forceinline__ void pull(const S* __restrict__ Fin, const S* __restr
 // only the low-order moments of the pulled populations.
 // seed: the node's rounding dither (dither_seed of its global index and the step) for
 // the stochastically rounded flow stores of the 16-bit forms; unused otherwise.
-template <typename S, int Q, bool UNIT = false>
+// IMPOSE (unit rates, FP32 and FP64): the stored state is moved to the u and T of
+// imposed[c] = (u_x, u_y, u_z, T), keeping the node's departure from equilibrium.
+template <typename S, int Q, bool UNIT = false, bool IMPOSE = false>
 __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15],
                                               typename Storage<S>::real (&g)[Q],
                                               S* __restrict__ Fout, S* __restrict__ Gout,
                                               float* __restrict__ Tout,
-                                              const ParamsOf<S>& p, int64_t c, uint32_t seed = 0) {
+                                              const ParamsOf<S>& p, int64_t c, uint32_t seed = 0,
+                                              const typename Storage<S>::real* __restrict__ imposed = nullptr) {
     using real = typename Storage<S>::real;
     using St = Storage<S>;
     const int64_t P = p.plane;
@@ -126,7 +129,20 @@ __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15]
         const real inv_rho = real(1) / (real(1) + dm.m0);
         UPow<real> u;
         Raw15<real> D;
-        flow_unit<real>(dm, Fx, Fy, Fz, r, inv_rho, u, D);
+        real Ts = T;  // the stored state's temperature and velocity
+        UPow<real> v;
+        if constexpr (IMPOSE) {
+            static_assert(!St::deviation, "the 16-bit forms impose in a pass of their own");
+            struct alignas(4 * sizeof(real)) Four {
+                real x, y, z, t;
+            };
+            const Four w = reinterpret_cast<const Four*>(imposed)[c];
+            Ts = w.t;
+            v = upow<real>(w.x, w.y, w.z);
+            flow_unit_imposed<real>(dm, Fx, Fy, Fz, r, inv_rho, u, v, D);
+        } else {
+            flow_unit<real>(dm, Fx, Fy, Fz, r, inv_rho, u, D);
+        }
         populations15<real>(D, f);  // f~ - w_a: the 16-bit forms store it as it is
 #pragma unroll
         for (int a = 0; a < 15; ++a) {
@@ -134,10 +150,12 @@ __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15]
             else Fout[a * P + c] = St::store(f[a] + p.wf[a], real(0));
         }
         if constexpr (Q == 15) {
-            thermal15_unit<real>(T, m0, mx, my, mz, u, r, D);
+            if constexpr (IMPOSE) thermal15_unit_imposed<real>(m0, mx, my, mz, u, r, Ts, v, D);
+            else thermal15_unit<real>(T, m0, mx, my, mz, u, r, D);
             populations15<real>(D, g);
         } else {
-            thermal7_unit<real>(T, m0, mx, my, mz, u, r, g);
+            if constexpr (IMPOSE) thermal7_unit_imposed<real>(m0, mx, my, mz, u, r, Ts, v, g);
+            else thermal7_unit<real>(T, m0, mx, my, mz, u, r, g);
         }
         if constexpr (St::deviation) Tout[c] = T;  // the reference of the stored deviations
 #pragma unroll
@@ -145,7 +163,7 @@ __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15]
             if constexpr (St::deviation)
                 Gout[a * P + c] = store16<S, St::sr_thermal>(g[a], dither_of(seed, 15 + a));
             else
-                Gout[a * P + c] = St::store(fmad(p.wg[a], T, g[a]), real(0));
+                Gout[a * P + c] = St::store(fmad(p.wg[a], Ts, g[a]), real(0));
         }
         return;
     }
@@ -182,12 +200,13 @@ __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15]
 // every thread.  Nodes touching a y or z wall run the generic pull.  The interior body
 // needs boundary == 0 (the cavity) and 15 * plane < 2^31 (32-bit node indices).
 // ---------------------------------------------------------------------------------
-template <typename S, int Q, bool INTERIOR, bool UNIT = false>
+template <typename S, int Q, bool INTERIOR, bool UNIT = false, bool IMPOSE = false>
 __device__ __forceinline__ void cavity_node(const S* __restrict__ Fin, const S* __restrict__ Gin,
                                             const float* __restrict__ Tin, S* __restrict__ Fout,
                                             S* __restrict__ Gout, float* __restrict__ Tout,
                                             const ParamsOf<S>& p, int i, int j, int k,
-                                            uint32_t step = 0) {
+                                            uint32_t step = 0,
+                                            const typename Storage<S>::real* __restrict__ imposed = nullptr) {
     using real = typename Storage<S>::real;
     using St = Storage<S>;
     const int nx = p.nx;
@@ -229,7 +248,7 @@ __device__ __forceinline__ void cavity_node(const S* __restrict__ Fin, const S* 
     }
     uint32_t seed = 0;
     if constexpr (St::deviation) seed = dither_seed((uint32_t)(p.cell0 + c), step);
-    collide_store<S, Q, UNIT>(f, g, Fout, Gout, Tout, p, c, seed);
+    collide_store<S, Q, UNIT, IMPOSE>(f, g, Fout, Gout, Tout, p, c, seed, imposed);
 }
 
 // Blocks per SM the single-precision kernels are built for: 7 for D3Q15 (at most 72

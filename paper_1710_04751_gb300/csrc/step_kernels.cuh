@@ -90,20 +90,23 @@ __global__ void __launch_bounds__(256) step_kernel(const S* __restrict__ Fin,
 // Cavity kernel: one block per x-row segment (blockIdx.y = j, blockIdx.z = k), so the
 // y/z wall tests are block-uniform.
 // ---------------------------------------------------------------------------------
-template <typename S, int Q, bool UNIT>
-__global__ void __launch_bounds__(128, (cavity_min_blocks<S, Q>()))
+template <typename S, int Q, bool UNIT, bool IMPOSE = false>
+__global__ void __launch_bounds__(128, (cavity_min_blocks<S, Q>() - (IMPOSE && cavity_min_blocks<S, Q>() > 1)))
     step_cavity_kernel(const S* __restrict__ Fin, const S* __restrict__ Gin,
                        const float* __restrict__ Tin, S* __restrict__ Fout,
                        S* __restrict__ Gout, float* __restrict__ Tout, ParamsOf<S> p,
-                       const unsigned* __restrict__ ctr_in, unsigned* __restrict__ ctr_out) {
+                       const unsigned* __restrict__ ctr_in, unsigned* __restrict__ ctr_out,
+                       const typename Storage<S>::real* __restrict__ imposed) {
     pdl_begin();
     const uint32_t step = step_of<S>(ctr_in, ctr_out);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y, k = blockIdx.z;
     if (i >= p.nx) return;
     const bool interior = j >= 1 && j + 1 < p.ny && k >= 1 && k + 1 < p.nz;
-    if (interior) cavity_node<S, Q, true, UNIT>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step);
-    else cavity_node<S, Q, false, UNIT>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step);
+    if (interior)
+        cavity_node<S, Q, true, UNIT, IMPOSE>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
+    else
+        cavity_node<S, Q, false, UNIT, IMPOSE>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
 }
 
 // ---------------------------------------------------------------------------------
@@ -282,6 +285,44 @@ bool launch_pair(const DevState& s, int cur, const ParamsOf<S>& p, cudaStream_t 
 }
 
 
+// Whether step_cavity_kernel takes the grid.
+template <typename real>
+bool cavity_kernel_fits(const DevParams<real>& p) {
+    return p.boundary == 0 && p.ny <= 65535 && p.nz <= 65535 && 15 * p.plane < (int64_t(1) << 31);
+}
+
+// Threads of a cavity-kernel block, along x.  FP64: one warp.  The two FP64 lanes per clock and
+// SM bound the kernel, so what counts is that every SM gets the same number of working warps:
+// at 32^3 a block of 128 threads per row held one working warp and the registers of four.
+// 42 -> 28 us a step at 32^3.  Single precision: the lanes of a row's last block that are left
+// idle cost nothing measurable (rows of 24, 64, 91 packed without gaps: 0.98-1.0x).
+template <typename S>
+constexpr int cavity_threads() {
+    return sizeof(typename Storage<S>::real) == 8 ? 32 : 128;
+}
+
+// One step of a cavity at unit rates whose result is moved to the u and T of imposed
+// ([ncell][4] = u_x, u_y, u_z, T, aligned to a quadruple); only where step_imposable says so.
+template <typename S>
+cudaError_t launch_step_imposed_as(const DevState& s, int cur, const ParamsOf<S>& p,
+                                   const typename Storage<S>::real* imposed, cudaStream_t st) {
+    const S* Fin = static_cast<const S*>(s.F[cur]);
+    const S* Gin = static_cast<const S*>(s.G[cur]);
+    S* Fout = static_cast<S*>(s.F[cur ^ 1]);
+    S* Gout = static_cast<S*>(s.G[cur ^ 1]);
+    const int bx = cavity_threads<S>();
+    const dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
+    const float* Tin = nullptr;
+    float* Tout = nullptr;
+    const unsigned* ctr_in = nullptr;
+    unsigned* ctr_out = nullptr;
+    if (s.Q == 15)
+        return launch_pdl(step_cavity_kernel<S, 15, true, true>, grid, dim3(bx), st, Fin, Gin, Tin, Fout, Gout,
+                          Tout, p, ctr_in, ctr_out, imposed);
+    return launch_pdl(step_cavity_kernel<S, 7, true, true>, grid, dim3(bx), st, Fin, Gin, Tin, Fout, Gout, Tout,
+                      p, ctr_in, ctr_out, imposed);
+}
+
 template <typename S, bool UNIT>
 cudaError_t launch_step_as(const DevState& s, int cur, const ParamsOf<S>& p, cudaStream_t st) {
     const S* Fin = static_cast<const S*>(s.F[cur]);
@@ -293,19 +334,15 @@ cudaError_t launch_step_as(const DevState& s, int cur, const ParamsOf<S>& p, cud
     if (launch_pair<S, UNIT>(s, cur, p, st)) return cudaGetLastError();
     const unsigned* ctr_in = s.step_ctr ? s.step_ctr + cur : nullptr;
     unsigned* ctr_out = s.step_ctr ? s.step_ctr + (cur ^ 1) : nullptr;
-    if (p.boundary == 0 && p.ny <= 65535 && p.nz <= 65535 && 15 * p.plane < (int64_t(1) << 31)) {
-        // FP64: one warp per block.  The two FP64 lanes per clock and SM bound the kernel, so
-        // what counts is that every SM gets the same number of working warps: at 32^3 a block of
-        // 128 threads per row held one working warp and the registers of four.  42 -> 28 us a
-        // step at 32^3.  Single precision: the lanes of a row's last block that are left idle
-        // cost nothing measurable (rows of 24, 64, 91 packed without gaps: 0.99-1.0x).
-        const int bx = sizeof(typename Storage<S>::real) == 8 ? 32 : 128;
+    if (cavity_kernel_fits(p)) {
+        const int bx = cavity_threads<S>();
         const dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
+        const typename Storage<S>::real* none = nullptr;
         if (s.Q == 15)
             return launch_pdl(step_cavity_kernel<S, 15, UNIT>, grid, dim3(bx), st, Fin, Gin, Tin, Fout, Gout,
-                              Tout, p, ctr_in, ctr_out);
+                              Tout, p, ctr_in, ctr_out, none);
         return launch_pdl(step_cavity_kernel<S, 7, UNIT>, grid, dim3(bx), st, Fin, Gin, Tin, Fout, Gout, Tout,
-                          p, ctr_in, ctr_out);
+                          p, ctr_in, ctr_out, none);
     }
     const int threads = 256;
     const int64_t blocks = (p.ncell + threads - 1) / threads;
