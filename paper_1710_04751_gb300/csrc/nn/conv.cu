@@ -55,6 +55,42 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, int bkc) {
     return bkc == 64 ? sdesc_k_sw128(saddr) : sdesc_k_sw64(saddr);
 }
 
+// Epilogue of 16 output channels col0.. of one voxel: bias + ReLU + BF16, or FP32.
+__device__ __forceinline__ void conv_store16(void* out, int N, int mode, const float* __restrict__ bias,
+                                             int row, int col0, float (&v)[16]) {
+    if (col0 >= N) return;
+    const bool whole = col0 + 16 <= N && (N % 8) == 0;  // 16-byte stores
+    if (mode == CONV_BIAS_RELU_BF16) {
+        __nv_bfloat16* C = static_cast<__nv_bfloat16*>(out) + (int64_t)row * N;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j] + (col0 + j < N ? bias[col0 + j] : 0.f), 0.f);
+        if (whole) {
+            uint4 pk[2];
+            __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(pk);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+            reinterpret_cast<uint4*>(C + col0)[0] = pk[0];
+            reinterpret_cast<uint4*>(C + col0)[1] = pk[1];
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (col0 + j < N) C[col0 + j] = __float2bfloat16_rn(v[j]);
+        }
+    } else {
+        float* C = static_cast<float*>(out) + (int64_t)row * N;
+        if (whole) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                reinterpret_cast<float4*>(C + col0)[j] =
+                    make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (col0 + j < N) C[col0 + j] = v[j];
+        }
+    }
+}
+
 template <int BN, int BKC>
 __global__ void __launch_bounds__(128, 1)
     conv_bf16_kernel(const __grid_constant__ CUtensorMap tmX,
@@ -148,39 +184,7 @@ __global__ void __launch_bounds__(128, 1)
         for (int c = 0; c < BN; c += 16) {
             float v[16];
             tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
-            const int col0 = n0 + c;
-            if (row >= args.M || col0 >= args.N) continue;
-            const bool whole = col0 + 16 <= args.N && (args.N % 8) == 0;  // 16-byte stores
-            if (args.mode == CONV_BIAS_RELU_BF16) {
-                __nv_bfloat16* C = static_cast<__nv_bfloat16*>(args.C) + (int64_t)row * args.N;
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    v[j] = fmaxf(v[j] + (col0 + j < args.N ? args.bias[col0 + j] : 0.f), 0.f);
-                if (whole) {
-                    uint4 pk[2];
-                    __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(pk);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                    reinterpret_cast<uint4*>(C + col0)[0] = pk[0];
-                    reinterpret_cast<uint4*>(C + col0)[1] = pk[1];
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (col0 + j < args.N) C[col0 + j] = __float2bfloat16_rn(v[j]);
-                }
-            } else {
-                float* C = static_cast<float*>(args.C) + (int64_t)row * args.N;
-                if (whole && (args.N % 4) == 0) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        reinterpret_cast<float4*>(C + col0)[j] =
-                            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (col0 + j < args.N) C[col0 + j] = v[j];
-                }
-            }
+            if (row < args.M) conv_store16(args.C, args.N, args.mode, args.bias, row, n0 + c, v);
         }
     }
     tc_fence_before();
@@ -189,49 +193,59 @@ __global__ void __launch_bounds__(128, 1)
 }
 
 // ---------------------------------------------------------------------------------
-// The same convolution with the input tile reused across the three ky taps (n >= 16).
-// A CTA computes MT consecutive M tiles (MT * 128 voxels: bx = n columns by MT * by rows of
-// one plane).  For each (kz, kx, channel chunk) one 5D box brings the MT * by + 2 rows
-// around them, shifted by kx - 1 in x and kz - 1 in z; the tile of output tile t and tap
-// ky is the 128-row window starting at row (t * by + ky) * bx of that box (whole x-rows,
-// so every window starts on a swizzle atom), multiplied into accumulator t with the
-// weights of tap (kz, ky, kx).  Each loaded byte serves up to 3 * MT * by / (MT * by + 2)
-// windows instead of one (2.4 at n = 64, MT = 4), cutting the operand traffic from L2 that
-// bounds the one-tile kernel.  Stage geometry is a runtime property of n and MT.
+// The same convolution with the three kx taps side by side in the MMA's N (16 <= n <= 128; the
+// kernel above takes the grids below and beyond).
+// An MMA of M = 128 voxels reads 4 KB of A from shared memory per 16 input channels whatever
+// its N, so at N = 32 output channels the operand reads (40 cycles) and not the 16 cycles of
+// tensor math bound the kernels above.  Here B holds the weights of kx = 0, 1, 2 of a (kz, ky)
+// row as 3 BN columns, and A is the UNSHIFTED x-row: the accumulator column kx BN + c of voxel
+// x is P_kx[x] = sum over (kz, ky, ci) of X[x] W[c][kz, ky, kx], and the epilogue adds
+//   Y[x] = P_0[x - 1] + P_1[x] + P_2[x + 1]
+// (P outside the row is the zero padding), the neighbours' values coming by warp shuffles and,
+// where an x-row spans several warps (n > 32), through shared memory.  A third of the A reads
+// and MMAs, each three times as wide.  A stage holds, of one kz and 32 input channels, the x-rows
+// of MT tiles plus one on either side (one 5D box, zero-filled outside the grid), and the tile of
+// tap ky is the 128-row window starting at row (t by + ky) n of that box: whole x-rows, so every
+// window starts on a swizzle atom, and each loaded row serves three ky taps.
 // ---------------------------------------------------------------------------------
-struct RowsArgs {
-    int M, N, n, chunks, cin;
-    int bx, by, mt;      // tile columns, rows per tile, tiles per CTA
-    int a_bytes;         // one stage's input box: (mt by + 2) bx BKC 2 bytes
-    int stage_bytes;     // a_bytes + 3 BN BKC 2, rounded up to 1024
+struct X3Args {
+    int N, n, chunks, cin;  // chunks of 32 input channels
+    int ntiles;             // tiles of BN output channels
+    int by, mt;             // rows per 128-voxel tile, tiles per CTA
+    int a_bytes;            // one stage's input box: (mt by + 2) n 64 bytes
+    int stage_bytes;        // a_bytes + 9 BN 64
     int stages;
-    uint32_t tmem_cols;  // mt BN, a power of two >= 32
+    uint32_t tmem_cols;     // mt 3 BN rounded up to a power of two
     int mode;
     void* C;
     const float* bias;
     int* err;
 };
 
-template <int BN, int BKC>
+template <int BN>
 __global__ void __launch_bounds__(128, 1)
-    conv_rows_kernel(const __grid_constant__ CUtensorMap tmX,
-                     const __grid_constant__ CUtensorMap tmW, RowsArgs args) {
-    extern __shared__ uint8_t rows_smem_raw[];
+    conv_x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
+                   X3Args args) {
+    extern __shared__ uint8_t x3_smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
-        (reinterpret_cast<uintptr_t>(rows_smem_raw) + 1023) & ~uintptr_t(1023));
+        (reinterpret_cast<uintptr_t>(x3_smem_raw) + 1023) & ~uintptr_t(1023));
     const int S = args.stages;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * args.stage_bytes);
     uint64_t* empty = full + S;
     uint64_t* done = empty + S;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     __shared__ volatile int failed;
-    constexpr int B_TILE = BN * BKC * 2;
+    __shared__ float edge[2][4][2][16];  // P_0 of a warp's last row, P_2 of its first
+    constexpr int W = 3 * BN, B_TILE = BN * 64;
 
-    if (*static_cast<volatile int*>(args.err) != 0) return;
+    if (*static_cast<volatile int*>(args.err) != 0) return;  // another CTA timed out
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int MT = args.mt;
-    const int m0 = blockIdx.x * MT * CBM, n0 = blockIdx.y * BN;
-    const int nkb = 9 * args.chunks;  // stages: (kz, kx, chunk)
+    const int MT = args.mt, n = args.n;
+    const int mg = blockIdx.x / args.ntiles, n0 = (blockIdx.x - mg * args.ntiles) * BN;
+    const int m0 = mg * MT * CBM;
+    const int y0 = (m0 / n) % n, z0 = (m0 / (n * n)) % n, b0 = m0 / (n * n * n);
+    const int kz0 = z0 == 0 ? 1 : 0, kz1 = z0 == n - 1 ? 2 : 3;  // planes inside the grid
+    const int nkb = (kz1 - kz0) * args.chunks;                   // stages: (kz, chunk)
 
     if (threadIdx.x == 0) {
         failed = 0;
@@ -250,9 +264,7 @@ __global__ void __launch_bounds__(128, 1)
 
     int issued = 0;
     if (warp == 0 && lane == 0) {
-        const int n = args.n;
-        const int y0 = (m0 / n) % n, z0 = (m0 / (n * n)) % n, b0 = m0 / (n * n * n);
-        int kz = 0, kx = 0, chunk = 0;
+        int kz = kz0, chunk = 0;
         for (int i = 0; i < nkb; ++i) {
             const int s = i % S;
             const uint32_t ph = (uint32_t)(i / S) & 1u;
@@ -262,25 +274,19 @@ __global__ void __launch_bounds__(128, 1)
             }
             if (failed) break;
             uint8_t* a = smem + s * args.stage_bytes;
-            mbar_expect_tx(full + s, (uint32_t)(args.a_bytes + 3 * B_TILE));
-            tma_load_5d(a, &tmX, full + s, chunk * BKC, kx - 1, y0 - 1, z0 + kz - 1, b0);
-            for (int ky = 0; ky < 3; ++ky) {
-                const int tap = (kz * 3 + ky) * 3 + kx;
-                tma_load_2d(a + args.a_bytes + ky * B_TILE, &tmW, full + s,
-                            (tap * args.chunks + chunk) * BKC, n0);
-            }
+            mbar_expect_tx(full + s, (uint32_t)(args.a_bytes + 9 * B_TILE));
+            tma_load_5d(a, &tmX, full + s, chunk * 32, 0, y0 - 1, z0 + kz - 1, b0);
+            for (int t = 0; t < 9; ++t)  // (ky, kx) of this kz
+                tma_load_2d(a + args.a_bytes + t * B_TILE, &tmW, full + s,
+                            (kz * 9 + t) * args.cin + chunk * 32, n0);
             ++issued;
             if (++chunk == args.chunks) {
                 chunk = 0;
-                if (++kx == 3) {
-                    kx = 0;
-                    ++kz;
-                }
+                ++kz;
             }
         }
     } else if (warp == 1 && lane == 0) {
-        const uint32_t idesc = idesc_bf16_f32(CBM, BN);
-        const int row_bytes = BKC * 2;
+        const uint32_t idesc = idesc_bf16_f32(CBM, W);
         for (int i = 0; i < nkb; ++i) {
             const int s = i % S;
             const uint32_t ph = (uint32_t)(i / S) & 1u;
@@ -291,68 +297,65 @@ __global__ void __launch_bounds__(128, 1)
             tc_fence_after();
             const uint32_t a = smem_u32(smem + s * args.stage_bytes), b = a + args.a_bytes;
             for (int t = 0; t < MT; ++t) {
-                for (int ky = 0; ky < 3; ++ky) {
-                    const uint32_t at = a + (uint32_t)((t * args.by + ky) * args.bx * row_bytes);
-                    const uint32_t bt = b + (uint32_t)(ky * B_TILE);
 #pragma unroll
-                    for (int kk = 0; kk < BKC / 16; ++kk)
-                        mma_bf16(tmem + (uint32_t)(t * BN), sdesc(at + kk * 32, BKC),
-                                 sdesc(bt + kk * 32, BKC), idesc, (i > 0 || ky > 0 || kk > 0) ? 1u : 0u);
+                for (int ky = 0; ky < 3; ++ky) {
+                    const uint32_t at = a + (uint32_t)((t * args.by + ky) * n * 64);
+                    const uint32_t bt = b + (uint32_t)(ky * 3 * B_TILE);
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk)
+                        mma_bf16(tmem + (uint32_t)(t * W), sdesc_k_sw64(at + kk * 32), sdesc_k_sw64(bt + kk * 32),
+                                 idesc, (i > 0 || ky > 0 || kk > 0) ? 1u : 0u);
                 }
             }
             mma_commit(empty + s);
         }
-        mma_commit(done);
+        mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
     }
     __syncwarp();
     if (!mbar_wait(done, 0, args.err, 3)) failed = 1;
     __syncthreads();
     const bool ok = !failed;
-    if (warp == 0 && lane == 0 && failed) {
+    if (warp == 0 && lane == 0 && failed) {  // let every started copy land
         for (int i = max(0, issued - S); i < issued; ++i)
             mbar_wait(full + (i % S), (uint32_t)(i / S) & 1u, args.err, 4);
     }
     tc_fence_after();
     if (ok) {
+        const int x = (warp * 32 + lane) & (n - 1);
+        const bool first = x == 0, last = x == n - 1;
+        int par = 0;
         for (int t = 0; t < MT; ++t) {
             const int row = m0 + t * CBM + warp * 32 + lane;
+            const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * W);
 #pragma unroll 1
-            for (int c = 0; c < BN; c += 16) {
-                float v[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * BN + c), v);
-                const int col0 = n0 + c;
-                if (row >= args.M || col0 >= args.N) continue;
-                const bool whole = col0 + 16 <= args.N && (args.N % 8) == 0;
-                if (args.mode == CONV_BIAS_RELU_BF16) {
-                    __nv_bfloat16* C = static_cast<__nv_bfloat16*>(args.C) + (int64_t)row * args.N;
+            for (int c = 0; c < BN; c += 16, par ^= 1) {
+                float p0[16], v[16], p2[16];
+                tmem_ld16_issue(base + (uint32_t)c, p0);
+                tmem_ld16_issue(base + (uint32_t)(BN + c), v);
+                tmem_ld16_issue(base + (uint32_t)(2 * BN + c), p2);
+                tmem_wait_ld();
+                tmem_landed(p0);
+                tmem_landed(v);
+                tmem_landed(p2);
+                if (n > 32) {  // block-uniform
+                    if (lane == 31) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        v[j] = fmaxf(v[j] + (col0 + j < args.N ? args.bias[col0 + j] : 0.f), 0.f);
-                    if (whole) {
-                        uint4 pk[2];
-                        __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(pk);
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                        reinterpret_cast<uint4*>(C + col0)[0] = pk[0];
-                        reinterpret_cast<uint4*>(C + col0)[1] = pk[1];
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (col0 + j < args.N) C[col0 + j] = __float2bfloat16_rn(v[j]);
+                        for (int j = 0; j < 16; ++j) edge[par][warp][0][j] = p0[j];
                     }
-                } else {
-                    float* C = static_cast<float*>(args.C) + (int64_t)row * args.N;
-                    if (whole && (args.N % 4) == 0) {
+                    if (lane == 0) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            reinterpret_cast<float4*>(C + col0)[j] =
-                                make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (col0 + j < args.N) C[col0 + j] = v[j];
+                        for (int j = 0; j < 16; ++j) edge[par][warp][1][j] = p2[j];
                     }
+                    __syncthreads();
                 }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    float l = __shfl_up_sync(0xffffffffu, p0[j], 1), r = __shfl_down_sync(0xffffffffu, p2[j], 1);
+                    if (lane == 0 && !first) l = edge[par][warp - 1][0][j];
+                    if (lane == 31 && !last) r = edge[par][warp + 1][1][j];
+                    v[j] += (first ? 0.f : l) + (last ? 0.f : r);
+                }
+                conv_store16(args.C, args.N, args.mode, args.bias, row, n0 + c, v);
             }
         }
     }
@@ -603,34 +606,22 @@ cudaError_t launch_conv(const CUtensorMap& tx, const CUtensorMap& tw, const Conv
     return cudaGetLastError();
 }
 
-constexpr int kRowsSmemBudget = 200 * 1024;
+constexpr int kX3Smem = 104 * 1024;     // stages of one of two CTAs on an SM
+constexpr int kX3SmemMax = 200 * 1024;  // of one alone
+constexpr int kSMs = 152;
 
-template <int BN, int BKC>
-cudaError_t launch_rows(const CUtensorMap& tx, const CUtensorMap& tw, const RowsArgs& a,
-                        cudaStream_t st) {
+template <int BN>
+cudaError_t launch_x3(const CUtensorMap& tx, const CUtensorMap& tw, const X3Args& a, int groups, cudaStream_t st) {
     static std::once_flag once;
     static cudaError_t attr = cudaSuccess;
     std::call_once(once, [] {
-        attr = cudaFuncSetAttribute(conv_rows_kernel<BN, BKC>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    1024 + kRowsSmemBudget + 256);
+        attr = cudaFuncSetAttribute(conv_x3_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    1024 + kX3SmemMax + 256);
     });
     if (attr != cudaSuccess) return attr;
     const size_t smem = 1024 + (size_t)a.stages * a.stage_bytes + 256;
-    const dim3 grid((a.M + a.mt * CBM - 1) / (a.mt * CBM), (a.N + BN - 1) / BN, 1);
-    conv_rows_kernel<BN, BKC><<<grid, 128, smem, st>>>(tx, tw, a);
+    conv_x3_kernel<BN><<<groups * a.ntiles, 128, smem, st>>>(tx, tw, a);
     return cudaGetLastError();
-}
-
-template <int BKC>
-cudaError_t launch_rows_bkc(const CUtensorMap& tx, const CUtensorMap& tw, const RowsArgs& a,
-                            int BN, cudaStream_t st) {
-    switch (BN) {
-    case 32: return launch_rows<32, BKC>(tx, tw, a, st);
-    case 64: return launch_rows<64, BKC>(tx, tw, a, st);
-    case 128: return launch_rows<128, BKC>(tx, tw, a, st);
-    default: return launch_rows<256, BKC>(tx, tw, a, st);
-    }
 }
 
 template <int BKC>
@@ -661,13 +652,6 @@ cudaError_t launch_wgrad(const CUtensorMap& tx, const CUtensorMap& tb, const Wgr
 
 }  // namespace
 
-// Tiles of >= 128 output channels at n >= 16 take the row-reuse kernel (conv_rows_kernel);
-// the rest the one-tile kernel.
-#ifndef LBM_CONV_ROWS
-#define LBM_CONV_ROWS 1
-#endif
-constexpr bool kConvRows = LBM_CONV_ROWS != 0;
-
 bool conv_implicit_supported(int n, int cin, int cout) {
     return cin % 32 == 0 && n >= 2 && n <= 256 && (n & (n - 1)) == 0 && cout >= 1 && cout <= 256;
 }
@@ -687,29 +671,39 @@ cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const _
     const int bb = 128 / (bx * by * bz);
     if (bx * by * bz * bb != 128) return cudaErrorInvalidValue;
     const int BN = cout <= 32 ? 32 : cout <= 64 ? 64 : cout <= 128 ? 128 : 256;
-    // the row-reuse kernel where it measured faster: tiles of 128 or more output channels
-    // (at 64 and fewer the tensor pipe's reads of the A operand from shared memory bound both
-    // kernels, and the one-tile kernel keeps more CTAs per SM)
-    if (kConvRows && BN >= 128 && n >= 16 && n <= 128) {
-        // tiles of whole x-rows of one plane, MT of them per CTA: as many as the tensor
-        // memory (MT BN columns) and two pipeline stages of shared memory allow
-        const int by1 = 128 / n;
-        const int b_bytes = 3 * BN * bkc * 2;
+    if (n >= 16 && n <= 128) {
+        // output channels per CTA: one tile up to 64, else tiles of 48 or 64 with less padding
+        const int bn = cout <= 16 ? 16 : cout <= 32 ? 32 : cout <= 48 ? 48 : cout <= 64 ? 64
+                     : (cout + 47) / 48 * 48 < (cout + 63) / 64 * 64 ? 48 : 64;
+        const int ntiles = (cout + bn - 1) / bn;
+        const int by1 = 128 / n, b_bytes = 9 * bn * 64;
+        const int64_t tiles = (int64_t)B * n * n * n / CBM;
+        auto stage_of = [&](int mt) { return (mt * by1 + 2) * n * 64 + b_bytes; };
+        // Two CTAs per SM, so that one computes while the other drains its accumulators: two
+        // stages in kX3Smem and at most half of the tensor memory each; within that the most
+        // tiles per CTA (they share the weights and the halo rows) that leave every SM a CTA.
+        // 64^3, batch 2, 96 -> 32 channels: 2 tiles 129 us a call, 1 tile 166, 4 tiles and one
+        // CTA per SM 153.
         int mt = 4;
-        while (mt > 1 && (mt * BN > 512 || mt * by1 > n ||
-                          2 * (((mt * by1 + 2) * n * bkc * 2 + b_bytes + 1023) / 1024 * 1024) > kRowsSmemBudget))
+        while (mt > 1 && (mt * 3 * bn > 256 || mt * by1 > n || 2 * stage_of(mt) > kX3Smem ||
+                          tiles / mt * ntiles < kSMs))
             mt >>= 1;
-        const int a_bytes = (mt * by1 + 2) * n * bkc * 2;
-        const int stage = (a_bytes + b_bytes + 1023) / 1024 * 1024;
-        if (2 * stage <= kRowsSmemBudget) {
-            const int stages = std::min(4, kRowsSmemBudget / stage);
-            CUtensorMap tx, tw;
-            if (!make_x_map(&tx, X, B, n, cin, bkc, n, mt * by1 + 2, 1, 1) ||
-                !make_w_map(&tw, W, cout, 27 * cin, ldw, bkc, BN))
-                return cudaErrorInvalidValue;
-            RowsArgs a{B * n * n * n, cout, n, cin / bkc, cin, n, by1, mt, a_bytes, stage, stages,
-                       (uint32_t)std::max(32, mt * BN), mode, out, bias, err};
-            return bkc == 64 ? launch_rows_bkc<64>(tx, tw, a, BN, st) : launch_rows_bkc<32>(tx, tw, a, BN, st);
+        const int stage = stage_of(mt);
+        const int stages = std::min(4, std::max(kX3Smem, kX3SmemMax * (2 * stage > kX3Smem)) / stage);
+        uint32_t cols = 32;
+        while ((int)cols < mt * 3 * bn) cols <<= 1;
+        CUtensorMap tx, tw;
+        if (!make_x_map(&tx, X, B, n, cin, 32, n, mt * by1 + 2, 1, 1) ||
+            !make_w_map(&tw, W, cout, 27 * cin, ldw, 32, bn))
+            return cudaErrorInvalidValue;
+        X3Args a{cout, n, cin / 32, cin, ntiles, by1, mt, (mt * by1 + 2) * n * 64, stage, stages, cols,
+                 mode, out, bias, err};
+        const int groups = (int)(tiles / mt);
+        switch (bn) {
+        case 16: return launch_x3<16>(tx, tw, a, groups, st);
+        case 32: return launch_x3<32>(tx, tw, a, groups, st);
+        case 48: return launch_x3<48>(tx, tw, a, groups, st);
+        default: return launch_x3<64>(tx, tw, a, groups, st);
         }
     }
     CUtensorMap tx, tw;
