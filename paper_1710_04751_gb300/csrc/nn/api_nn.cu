@@ -4,21 +4,22 @@
 #include "../context.h"
 #include "lbm_net.h"
 #include "nn.h"
+#include "tc.cuh"
 
 using namespace lbm;
 
 namespace {
 
-// Per-device error word the network kernels write on a timeout.
-__device__ int nn_error_word;
+// Per-device error cell the network kernels write on a timeout.
+__device__ nn::ErrorCell nn_error_cell;
 
 // Operand and output of the timeout diagnostic (nothing reads the operand; nothing is
 // stored to the output).
 __device__ __align__(128) __nv_bfloat16 nn_probe_operand[128 * 64];
 __device__ __align__(128) float nn_probe_out[128 * 32];
 
-// The device's error word and its mirror in page-locked host memory, into which finish()
-// copies the word behind the stream's work (one pair per device for the process's life).
+// The device's error cell and its mirror in page-locked host memory (one pair per device for the
+// process's life).
 struct ErrorWord {
     int* dev;
     int* host;
@@ -30,22 +31,28 @@ ErrorWord* error_word() {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
     std::lock_guard<std::mutex> g(mu);
-    if (!words[dev].dev) {
-        void* p = nullptr;
-        if (!words[dev].host && cudaMallocHost(&words[dev].host, sizeof(int)) != cudaSuccess) return nullptr;
-        if (cudaGetSymbolAddress(&p, nn_error_word) != cudaSuccess) return nullptr;
-        words[dev].dev = static_cast<int*>(p);
+    ErrorWord& w = words[dev];
+    if (!w.dev) {
+        void* cell = nullptr;
+        nn::ErrorCell init{};
+        if (!w.host && cudaHostAlloc(&w.host, sizeof(int), cudaHostAllocMapped) != cudaSuccess) return nullptr;
+        *w.host = 0;
+        if (cudaHostGetDevicePointer(&init.mirror, w.host, 0) != cudaSuccess ||
+            cudaGetSymbolAddress(&cell, nn_error_cell) != cudaSuccess ||
+            cudaMemcpy(cell, &init, sizeof init, cudaMemcpyHostToDevice) != cudaSuccess)
+            return nullptr;
+        w.dev = static_cast<int*>(cell);
     }
-    return &words[dev];
+    return &w;
 }
 
 // Waits for the stream and turns a recorded kernel timeout into LBM_ETIMEOUT.
 int finish(cudaStream_t st, ErrorWord* err) {
-    if (cudaMemcpyAsync(err->host, err->dev, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        return record_error(nullptr, LBM_ECUDA, "reading the network error word failed%s");
     int rc = wait_stream_for(st, 600.0, nullptr);
     if (rc != LBM_OK) return rc;
-    if (*static_cast<volatile int*>(err->host) != 0) {
+    volatile int* word = err->host;
+    if (*word != 0) {
+        *word = 0;
         cudaMemset(err->dev, 0, sizeof(int));
         return record_error(nullptr, LBM_ETIMEOUT, "a wait inside a tensor-core kernel timed out%s");
     }

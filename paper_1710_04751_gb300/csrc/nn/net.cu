@@ -27,6 +27,7 @@
 #include "../context.h"
 #include "lbm_net.h"
 #include "nn.h"
+#include "tc.cuh"
 
 using namespace lbm;
 using namespace lbm::nn;
@@ -69,7 +70,7 @@ struct lbm_net {
     double* partd;      // per-block partial sums of the loss
     double* loss;
     int* err;
-    double* host;       // page-locked: the loss, then the error word, read behind each call's work
+    double* host;       // page-locked: the loss read behind a call's work, then the error cell's mirror
     void* arena;
     size_t arena_bytes;
     int step;
@@ -408,15 +409,14 @@ int update(lbm_net* N) {
     return LBM_OK;
 }
 
-// The bounded wait, with the error word (and the loss) copied behind the stream's work into
-// page-locked memory first, so that one wait covers both.
+// The bounded wait, with the loss copied behind the stream's work into page-locked memory first.
 int wait_net(lbm_net* N, double* loss = nullptr) {
-    int* word = reinterpret_cast<int*>(N->host + 1);
-    NET_CUDA(N, cudaMemcpyAsync(word, N->err, sizeof(int), cudaMemcpyDeviceToHost, N->stream));
     if (loss) NET_CUDA(N, cudaMemcpyAsync(N->host, N->loss, sizeof(double), cudaMemcpyDeviceToHost, N->stream));
     int rc = wait_stream_for(N->stream, 600.0, &N->msg);
     if (rc != LBM_OK) return rc;
+    volatile int* word = reinterpret_cast<int*>(N->host + 1);
     if (*word) {
+        *word = 0;
         cudaMemset(N->err, 0, sizeof(int));
         return nfail(N, LBM_ETIMEOUT, "a wait inside a tensor-core kernel timed out%s");
     }
@@ -466,6 +466,7 @@ extern "C" void lbm_net_destroy(lbm_net* N) {
     if (!N) return;
     wait_stream_for(N->stream, 600.0, nullptr);
     if (N->arena) cudaFree(N->arena);
+    if (N->err) cudaFree(N->err);
     if (N->host) cudaFreeHost(N->host);
     delete N;
 }
@@ -518,9 +519,16 @@ extern "C" int lbm_net_create(const lbm_net_config* cfg, lbm_net** out) {
         return nfail(nullptr, LBM_ENOMEM, "cudaMalloc of the network failed: %s", cudaGetErrorString(e));
     }
     carve(N, static_cast<char*>(N->arena));
-    e = cudaMalloc(&N->err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMallocHost(&N->host, 2 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemset(N->err, 0, sizeof(int));
+    ErrorCell cell{};
+    e = cudaMalloc(&N->err, sizeof cell);
+    if (e == cudaSuccess) e = cudaHostAlloc(&N->host, 2 * sizeof(double), cudaHostAllocMapped);
+    if (e == cudaSuccess) {
+        N->host[1] = 0.0;
+        double* mirror = nullptr;
+        e = cudaHostGetDevicePointer(&mirror, N->host, 0);
+        cell.mirror = reinterpret_cast<int*>(mirror + 1);
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(N->err, &cell, sizeof cell, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(N->arena, 0, N->arena_bytes);  // zero moments
     if (e != cudaSuccess) {
         lbm_net_destroy(N);

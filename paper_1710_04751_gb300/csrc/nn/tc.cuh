@@ -45,9 +45,24 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
+// The error cell of the kernels' bounded waits.  Kernels get a pointer to `code` and, on a
+// timeout, write the code there (other CTAs poll it) and through `mirror` into page-locked host
+// memory, which the host reads once the kernel is done: no copy after every call.
+struct ErrorCell {
+    int code, pad;
+    int* mirror;
+};
+__device__ __forceinline__ void record_timeout(int* err, int code) {
+    atomicExch(err, code);
+    if (int* const m = reinterpret_cast<ErrorCell*>(err)->mirror) {
+        *static_cast<volatile int*>(m) = code;
+        __threadfence_system();
+    }
+}
+
 // Waits for the phase of `parity` to complete, for at most `limit_ns` nanoseconds, or
 // until *abort (another thread of the CTA gave up) is set; on timeout records `code` in
-// *err and returns false.
+// the error cell at err and returns false.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* err, int code,
                                           const volatile int* abort = nullptr,
                                           uint64_t limit_ns = 2000000000ull) {
@@ -58,7 +73,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
             if (mbar_try_wait(bar, parity)) return true;
         if (abort && *abort) return false;
         if (global_ns() - t0 > limit_ns) {
-            atomicExch(err, code);
+            record_timeout(err, code);
             return false;
         }
     }
