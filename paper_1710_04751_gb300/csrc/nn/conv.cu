@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(128, 1)
     constexpr int W = 3 * BN, B_TILE = BN * 64;
 
     if (*static_cast<volatile int*>(args.err) != 0) return;  // another CTA timed out
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int MT = args.mt, n = args.n;
     const int mg = blockIdx.x / args.ntiles, n0 = (blockIdx.x - mg * args.ntiles) * BN;
     const int m0 = mg * MT * CBM;
@@ -263,53 +263,62 @@ __global__ void __launch_bounds__(128, 1)
     const uint32_t tmem = *tmem_slot;
 
     int issued = 0;
-    if (warp == 0 && lane == 0) {
-        int kz = kz0, chunk = 0;
+    if (warp == 0) {
+        const bool elected = elect_lane();
+        int kz = kz0, chunk = 0, s = 0;
+        uint32_t ph = 1;  // parity of the slot's last release
         for (int i = 0; i < nkb; ++i) {
-            const int s = i % S;
-            const uint32_t ph = (uint32_t)(i / S) & 1u;
-            if (i >= S && !mbar_wait(empty + s, ph ^ 1u, args.err, 1, &failed)) {
+            if (i >= S && !mbar_wait_warp(empty + s, ph, args.err, 1, &failed)) {
                 failed = 1;
                 break;
             }
-            if (failed) break;
             uint8_t* a = smem + s * args.stage_bytes;
-            mbar_expect_tx(full + s, (uint32_t)(args.a_bytes + 9 * B_TILE));
-            tma_load_5d(a, &tmX, full + s, chunk * 32, 0, y0 - 1, z0 + kz - 1, b0);
-            for (int t = 0; t < 9; ++t)  // (ky, kx) of this kz
-                tma_load_2d(a + args.a_bytes + t * B_TILE, &tmW, full + s,
-                            (kz * 9 + t) * args.cin + chunk * 32, n0);
+            if (elected) {
+                mbar_expect_tx(full + s, (uint32_t)(args.a_bytes + 9 * B_TILE));
+                tma_load_5d(a, &tmX, full + s, chunk * 32, 0, y0 - 1, z0 + kz - 1, b0);
+#pragma unroll
+                for (int t = 0; t < 9; ++t)  // (ky, kx) of this kz
+                    tma_load_2d(a + args.a_bytes + t * B_TILE, &tmW, full + s,
+                                (kz * 9 + t) * args.cin + chunk * 32, n0);
+            }
             ++issued;
+            if (++s == S) s = 0, ph ^= 1u;
             if (++chunk == args.chunks) {
                 chunk = 0;
                 ++kz;
             }
         }
-    } else if (warp == 1 && lane == 0) {
-        const uint32_t idesc = idesc_bf16_f32(CBM, W);
+    } else if (warp == 1) {
+        const bool elected = elect_lane();
+        const uint32_t idesc = idesc_bf16_f32(CBM, W), dhi = (uint32_t)(sdesc_k_sw64(0) >> 32);
+        const uint32_t window = (uint32_t)(n * 64 >> 4);
+        int s = 0;
+        uint32_t ph = 0;
         for (int i = 0; i < nkb; ++i) {
-            const int s = i % S;
-            const uint32_t ph = (uint32_t)(i / S) & 1u;
-            if (failed || !mbar_wait(full + s, ph, args.err, 2, &failed)) {
+            if (!mbar_wait_warp(full + s, ph, args.err, 2, &failed)) {
                 failed = 1;
                 break;
             }
             tc_fence_after();
-            const uint32_t a = smem_u32(smem + s * args.stage_bytes), b = a + args.a_bytes;
-            for (int t = 0; t < MT; ++t) {
+            const uint32_t alo = (uint32_t)sdesc_k_sw64(smem_u32(smem + s * args.stage_bytes));
+            const uint32_t blo = (uint32_t)sdesc_k_sw64(smem_u32(smem + s * args.stage_bytes) + args.a_bytes);
+            if (elected) {
+              for (int t = 0; t < MT; ++t) {
 #pragma unroll
-                for (int ky = 0; ky < 3; ++ky) {
-                    const uint32_t at = a + (uint32_t)((t * args.by + ky) * n * 64);
-                    const uint32_t bt = b + (uint32_t)(ky * 3 * B_TILE);
+                for (int ky = 0; ky < 3; ++ky) {  // the window of tap ky: t 128 + ky n rows of 64 bytes on
+                    const uint32_t at = alo + (uint32_t)(t * (CBM * 64 >> 4)) + (uint32_t)ky * window;
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk)
-                        mma_bf16(tmem + (uint32_t)(t * W), sdesc_k_sw64(at + kk * 32), sdesc_k_sw64(bt + kk * 32),
-                                 idesc, (i > 0 || ky > 0 || kk > 0) ? 1u : 0u);
+                        mma_bf16_halves(tmem + (uint32_t)(t * W), at + kk * 2, dhi,
+                                        blo + (uint32_t)(ky * (3 * B_TILE >> 4)) + kk * 2, dhi, idesc,
+                                        (i > 0 || ky > 0 || kk > 0) ? 1u : 0u);
                 }
+              }
+              mma_commit(empty + s);
             }
-            mma_commit(empty + s);
+            if (++s == S) s = 0, ph ^= 1u;
         }
-        mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
+        if (elected) mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
     }
     __syncwarp();
     if (!mbar_wait(done, 0, args.err, 3)) failed = 1;

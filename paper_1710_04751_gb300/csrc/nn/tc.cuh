@@ -79,6 +79,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* e
     }
 }
 
+// The warp's index, and one elected lane of the warp, as values the compiler knows to be the
+// same across the warp.  TMA and MMA instructions take their operands from uniform registers:
+// in a branch on threadIdx every operand of every instruction is first moved there, some 100
+// (MMA) to 200 (TMA) cycles an instruction; a loop that the whole warp runs keeps them there,
+// and only the instruction itself is the elected lane's.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ bool elect_lane() {
+    uint32_t e;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(e));
+    return e != 0;
+}
+// mbar_wait by a whole warp: every lane's answer is the same.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, int code,
+                                               const volatile int* abort) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code, abort));
+}
+
 // 2D tiled TMA load of the box at (c0 = innermost element, c1 = row) into shared memory,
 // completing `bytes` on the barrier.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar,
@@ -131,6 +152,22 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// The same with each descriptor in two halves: the upper one (strides and layout) does not change
+// over an operand, and the lower one moves by an address step >> 4, so that the issuing thread
+// spends an addition per operand and MMA.  (A thread that builds 64-bit descriptors from
+// runtime strides for every MMA takes longer than a narrow MMA does.)
+__device__ __forceinline__ void mma_bf16_halves(uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                                uint32_t bhi, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 
