@@ -599,6 +599,252 @@ __global__ void __launch_bounds__(128, 1)
     if (warp == 0) tmem_dealloc(tmem, L::TMEM_COLS);
 }
 
+// ---------------------------------------------------------------------------------
+// The weight gradient with the nine (ky, kx) taps side by side in N (n >= 16, up to 64 output
+// channels).  With the tap's shift on the other operand,
+//   dW^T[kz, ky, kx][ci][co] = sum over u of X[u + kz][ci] dZ[u - (ky, kx)][co],
+// one A operand -- 64 voxels of X, four chunks of (kz, 32 channels) as the M tile's rows --
+// serves nine taps: for each ky one MMA of M = 128, N = 96 (kx, 32 output channels).  The kernel
+// above reads 4 KB of A from shared memory per MMA of N = 32, and every A byte from L2 once per
+// tap.  The kx shifts of dZ are three TMA boxes (zero-filled outside the grid); the ky shifts
+// come from the neighbouring x-rows: a slot of the ring holds the X rows y0 .. y0 + RB - 1 of a
+// block of 64 voxels and the dZ rows one further on, y0 + 1 .. y0 + RB, and the MMAs take the dZ
+// rows y0 - 1 .. y0 + RB from this slot and the one or two before it, so that each dZ row is
+// loaded once per kx.  A run of blocks that starts (at a plane's or the range's first block)
+// is led in by slots with dZ rows only.
+// The accumulators fill 288 tensor-memory columns: a CTA holds one M tile of 32 output
+// channels and a range of the blocks; where that leaves SMs idle, two CTAs of a cluster share a
+// range and the second adds its sums to the first's through distributed shared memory (a fixed
+// order).
+// ---------------------------------------------------------------------------------
+constexpr int W9_N = 96;                    // columns of one ky: 3 kx of 32 output channels
+constexpr int W9_ROWS = 64 * 64;            // bytes of 64 voxels of 32 channels
+constexpr int W9_SLOT = 7 * W9_ROWS;        // four chunks of X, three copies of dZ
+constexpr int W9_SLOTS = 7;
+constexpr int W9_SUM = 128 * 3 * W9_N * 4;  // bytes of one CTA's accumulators
+static_assert(W9_SLOTS * W9_SLOT >= W9_SUM, "the pair's sums go where the ring was");
+
+struct Wgrad9Args {
+    int N, cin, n;       // output channels, input channels, grid edge
+    int segs, run;       // 64-voxel segments of an x-row, blocks of a run (the rows of one
+                         // segment of one plane)
+    int total, per;      // blocks (64 voxels each) in all and per CTA
+    int Mrows;           // rows of a workspace slice (the padded 27 cin)
+    int pair;            // two CTAs of a cluster share a slice
+    float* ws;           // [slices][Mrows][N]
+    int* err;
+};
+
+// Walks a CTA's ring slots: `lead` slots before the first block of the range and of every run,
+// then the blocks, each at (b, z, seg, y): sample, plane, x-segment and block of its run.
+struct W9Walk {
+    int count, run, lead, segs, n;  // count: blocks still to come
+    int b, z, seg, y, left;         // left: lead-in slots still to come before this block
+    __device__ W9Walk(int first, int count_, int run_, int lead_, int segs_, int n_)
+        : count(count_), run(run_), lead(lead_), segs(segs_), n(n_), left(lead_) {
+        const int r = first / run, pl = r / segs;
+        y = first - r * run;
+        seg = r - pl * segs;
+        b = pl / n;
+        z = pl - b * n;
+    }
+    __device__ bool more() const { return count > 0; }
+    __device__ bool data() const { return left == 0; }  // a block's slot, not a lead-in
+    __device__ void next() {
+        if (left > 0) {
+            --left;
+            return;
+        }
+        --count;
+        if (++y < run) return;
+        y = 0, left = lead;
+        if (++seg < segs) return;
+        seg = 0;
+        if (++z == n) z = 0, ++b;
+    }
+};
+
+// RB: x-rows of a 64-voxel block: 64 / n, or 1.
+template <int RB>
+__global__ void __launch_bounds__(128, 1)
+    conv_wgrad9_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmZ,
+                       Wgrad9Args args) {
+    constexpr int S = W9_SLOTS;
+    extern __shared__ uint8_t w9_smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>(
+        (reinterpret_cast<uintptr_t>(w9_smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * W9_SLOT);
+    uint64_t* empty = full + S;
+    uint64_t* done = empty + S;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    __shared__ volatile int failed;
+
+    const int warp = warp_index(), lane = threadIdx.x & 31;
+    const int slice = args.pair ? blockIdx.x >> 1 : blockIdx.x;
+    const uint32_t rank = args.pair ? cluster_rank() : 0u;
+    const int mt = blockIdx.y, n0 = blockIdx.z * 32, n = args.n;
+    const int first = blockIdx.x * args.per;  // the pair's CTAs take consecutive ranges
+    const int nst = max(0, min(args.per, args.total - first));
+    constexpr int lead = RB == 1 ? 2 : 1;
+    const int gpt = args.cin >> 5;            // channel groups per kz
+
+    if (threadIdx.x == 0) {
+        // another CTA timed out: nothing is loaded or stored, but the pair's barriers are kept
+        failed = *static_cast<volatile int*>(args.err) != 0;
+        for (int s = 0; s < S; ++s) {
+            mbar_init(full + s, 1);
+            mbar_init(empty + s, 1);
+        }
+        mbar_init(done, 1);
+        mbar_fence_init();
+    }
+    if (warp == 0) tmem_alloc(tmem_slot, 512);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    int issued = 0;
+    if (warp == 0) {
+        const bool elected = elect_lane();
+        int gz[4], gc[4];  // kz - 1 and first channel of the M tile's chunks
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = mt * 4 + q, kz = c / gpt;
+            gz[q] = kz < 3 ? kz - 1 : 0;
+            gc[q] = kz < 3 ? (c - kz * gpt) * 32 : args.cin;  // past the last chunk: zeros
+        }
+        W9Walk w(first, nst, args.run, lead, args.segs, n);
+        int s = 0;
+        uint32_t ph = 1;  // parity of the slot's last release
+        for (int i = 0; w.more(); ++i, w.next()) {
+            if (i >= S && !mbar_wait_warp(empty + s, ph, args.err, 1, &failed)) {
+                failed = 1;
+                break;
+            }
+            uint8_t* a = smem + s * W9_SLOT;
+            const int x0 = w.seg * 64, y0 = w.y * RB, yz = y0 + 1 - w.left * RB;  // dZ rows yz .. yz + RB - 1
+            if (elected) {
+                mbar_expect_tx(full + s, (w.data() ? 7 : 3) * W9_ROWS);
+                if (w.data()) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        tma_load_5d(a + q * W9_ROWS, &tmX, full + s, gc[q], x0, y0, w.z + gz[q], w.b);
+                }
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx)
+                    tma_load_5d(a + (4 + kx) * W9_ROWS, &tmZ, full + s, n0, x0 + 1 - kx, yz, w.z, w.b);
+            }
+            ++issued;
+            if (++s == S) s = 0, ph ^= 1u;
+        }
+    } else if (nst > 0 && warp == 1) {
+        const bool elected = elect_lane();
+        const uint32_t idesc = idesc_bf16_f32_mn(CBM, W9_N);
+        const uint32_t ahi = (uint32_t)(sdesc_mn(0, W9_ROWS, 512, 4) >> 32);
+        const uint32_t ring = (uint32_t)sdesc_mn(smem_u32(smem), W9_ROWS, 512, 4);
+        uint32_t acc = 0, z[3] = {ring, ring, ring};  // dZ of this slot, of the one before, of two before
+        W9Walk w(first, nst, args.run, lead, args.segs, n);
+        int s = 0, s1 = S - 1, s2 = S - 2;  // this slot and the ones before
+        uint32_t ph = 0;
+        for (int i = 0; w.more(); ++i, w.next()) {
+            if (!mbar_wait_warp(full + s, ph, args.err, 2, &failed)) {
+                failed = 1;
+                break;
+            }
+            const uint32_t a = ring + (uint32_t)(s * (W9_SLOT >> 4));
+            z[2] = z[1], z[1] = z[0], z[0] = a + (4 * W9_ROWS >> 4);
+            tc_fence_after();
+            if (elected && w.data()) {
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {  // K = 16 per MMA: two atoms of 8 voxels
+                    constexpr int line = 64 / RB * 64;  // bytes of an x-row of the block
+                    const int row = kk * RB / 4;        // x-row of the block
+#pragma unroll
+                    for (int ky = 0; ky < 3; ++ky) {
+                        // dZ row y0 + row - (ky - 1): place d = row - ky of this slot, or of one before
+                        const int back = row >= ky ? 0 : (ky - row + RB - 1) / RB;
+                        const int d = row - ky + back * RB;
+                        mma_bf16_halves(tmem + (uint32_t)(ky * W9_N), a + kk * 64, ahi,
+                                        z[back] + (uint32_t)(((d - row) * line + kk * 1024) >> 4), ahi, idesc, acc);
+                    }
+                    acc = 1;
+                }
+            }
+            if (elected && i >= lead) mma_commit(empty + (lead == 2 ? s2 : s1));  // its dZ rows are used up
+            s2 = s1, s1 = s;
+            if (++s == S) s = 0, ph ^= 1u;
+        }
+        if (elected) mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
+    }
+    __syncwarp();
+    if (nst > 0 && !mbar_wait(done, 0, args.err, 3)) failed = 1;
+    __syncthreads();
+    if (warp == 0 && lane == 0 && failed) {  // let every started copy land
+        for (int i = max(0, issued - S); i < issued; ++i)
+            mbar_wait(full + (i % S), (uint32_t)(i / S) & 1u, args.err, 4);
+    }
+    __syncwarp();
+    tc_fence_after();
+    const uint32_t lanes = tmem + ((uint32_t)(warp * 32) << 16);
+    float4* sum = reinterpret_cast<float4*>(smem);  // [column / 4][128 rows]
+    if (args.pair) {
+        cluster_sync();  // both pipelines are done with their shared memory
+        if (rank == 1 && !failed) {
+            const uint32_t peer = cluster_map(smem_u32(smem), 0);
+#pragma unroll 1
+            for (int c = 0; c < 3 * W9_N; c += 16) {
+                float v[16];
+                tmem_ld16(lanes + (uint32_t)c, v);
+                if (nst == 0) {  // nothing accumulated
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] = 0.f;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    cluster_store4(peer + (uint32_t)((((c >> 2) + j) * 128 + threadIdx.x) * 16),
+                                   make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
+            }
+        }
+        cluster_sync();
+    }
+    const bool ok = rank == 0 && nst > 0 && !failed && *static_cast<volatile int*>(args.err) == 0;
+    const int chunk = mt * 4 + warp, kz = chunk / gpt;  // this warp's rows: one chunk
+    if (ok && kz < 3) {
+        const int ci = (chunk - kz * gpt) * 32 + lane;
+        float* slab = args.ws + (int64_t)slice * args.Mrows * args.N;
+#pragma unroll 1
+        for (int c = 0; c < 3 * W9_N; c += 16) {
+            float v[16];
+            tmem_ld16(lanes + (uint32_t)c, v);
+            if (args.pair) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float4 w = sum[((c >> 2) + j) * 128 + threadIdx.x];
+                    v[4 * j] += w.x;
+                    v[4 * j + 1] += w.y;
+                    v[4 * j + 2] += w.z;
+                    v[4 * j + 3] += w.w;
+                }
+            }
+            const int t = c >> 5, col0 = n0 + (c & 31);  // tap within kz (ky 3 + kx)
+            float* C = slab + (int64_t)((kz * 9 + t) * args.cin + ci) * args.N + col0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)  // N is a multiple of 8: whole quadruples
+                if (col0 + 4 * j < args.N)
+                    reinterpret_cast<float4*>(C)[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        }
+    }
+    if (ok && mt == 0) {  // the padding rows
+        float* pad = args.ws + ((int64_t)slice * args.Mrows + 27 * args.cin) * args.N;
+        for (int e = threadIdx.x; e < (args.Mrows - 27 * args.cin) * 32; e += 128)
+            if (n0 + (e & 31) < args.N) pad[(int64_t)(e >> 5) * args.N + n0 + (e & 31)] = 0.f;
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
 template <int BN, int BKC>
 cudaError_t launch_conv(const CUtensorMap& tx, const CUtensorMap& tw, const ConvArgs& a,
                         cudaStream_t st) {
@@ -723,6 +969,57 @@ cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const _
     return bkc == 64 ? launch_conv_bkc<64>(tx, tw, a, BN, st) : launch_conv_bkc<32>(tx, tw, a, BN, st);
 }
 
+// The nine-tap weight gradient: the slices (at most max_slices) and whether CTAs go in pairs.
+// The tensor core's FP32 accumulation truncates, so the length of its chains shows in the
+// result: about 7e-10 of relative error per voxel of a chain.  A chain may be up to 1.15 times
+// as long as max_slices make it; two chains of half the length may take its place up to
+// kPairChain voxels, beyond which that would move a result by 2e-5.  Among these the choice
+// that leaves the least work to the busiest SM.
+constexpr int kPairChain = 38400;
+cudaError_t launch_wgrad9(const __nv_bfloat16* X, int B, int n, int cin, const __nv_bfloat16* dZ, int cout, int Kp,
+                          float* ws, int max_slices, int* slices, int* err, cudaStream_t st) {
+    const int total = (int)((int64_t)B * n * n * n / 64);
+    const int mtiles = (3 * (cin / 32) + 3) / 4, ntiles = (cout + 31) / 32, tiles = mtiles * ntiles;
+    max_slices = std::min(max_slices, total);
+    int best_s = max_slices, best_c = 1;
+    int64_t best = INT64_MAX;
+    for (int c = 1; c <= ((int64_t)total * 64 <= (int64_t)kPairChain * max_slices ? 2 : 1); ++c)
+        for (int s = max_slices; s >= 1 && 100 * max_slices <= 115 * s; --s) {
+            const int64_t waves = ((int64_t)tiles * s * c + kSMs - 1) / kSMs;
+            const int64_t t = waves * ((total + s * c - 1) / (s * c) + 8);  // 8: prologue and drain
+            if (t < best) best = t, best_s = s, best_c = c;
+        }
+    const int per = (total + best_s * best_c - 1) / (best_s * best_c);
+    *slices = (total + per * best_c - 1) / (per * best_c);  // every slice has work in its first CTA
+    constexpr int smem = 1024 + W9_SLOTS * W9_SLOT + 256;
+    const auto kernel = n == 16 ? conv_wgrad9_kernel<4> : n == 32 ? conv_wgrad9_kernel<2> : conv_wgrad9_kernel<1>;
+    static std::once_flag once;
+    static cudaError_t attr = cudaSuccess;
+    std::call_once(once, [] {
+        for (const auto k : {conv_wgrad9_kernel<4>, conv_wgrad9_kernel<2>, conv_wgrad9_kernel<1>})
+            if (attr == cudaSuccess) attr = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    });
+    if (attr != cudaSuccess) return attr;
+    const int bx = n < 64 ? n : 64, RB = 64 / bx, segs = n / bx;
+    CUtensorMap tx, tz;
+    if (!make_x_map(&tx, X, B, n, cin, 32, bx, RB, 1, 1) || !make_x_map(&tz, dZ, B, n, cout, 32, bx, RB, 1, 1))
+        return cudaErrorInvalidValue;
+    const Wgrad9Args a{cout, cin, n, segs, n / RB, total, per, Kp, best_c == 2, ws, err};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(*slices * best_c), (unsigned)mtiles, (unsigned)ntiles);
+    cfg.blockDim = dim3(128);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)best_c;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = best_c == 2 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, tx, tz, a);
+}
+
 bool conv_wgrad_implicit_supported(int B, int n, int cin, int cout) {
     const int64_t M = (int64_t)B * n * n * n;
     return n >= 2 && n <= 256 && (n & (n - 1)) == 0 && cin % 32 == 0 && cout >= 8 && cout <= 256 &&
@@ -741,6 +1038,16 @@ cudaError_t conv_wgrad_implicit(const __nv_bfloat16* X, int B, int n, int cin, c
     const int used = (kblocks + per - 1) / per;
     const int mtiles = (Kp + CBM - 1) / CBM;
     if ((size_t)used * Kp * cout > ws_floats) return cudaErrorInvalidValue;
+    // The nine-tap form where it measured faster (calls with the host wait, us, one-tap / nine-tap):
+    // 64^3 batch 2, 96 -> 32 channels 286 / 190 and 32 -> 32 136 / 108, 32^3 batch 2, 192 -> 64
+    // 117 / 101; below that its long ramp shows: 32^3, 64 -> 64 79 / 82, 16^3 batch 4, 64 -> 48
+    // 64 / 75.  More than 64 output channels fill the one-tap form's MMAs.
+    if (n >= 16 && cout <= 64 && M * cin >= (int64_t(1) << 23)) {
+        int slices = 0;
+        const cudaError_t e = launch_wgrad9(X, B, n, cin, dZ, cout, Kp, ws, used, &slices, err, st);
+        if (e != cudaSuccess) return e;
+        return add_splits(ws, slices, Kp, cout, cout, dWT, accumulate, st);
+    }
     // the 64-voxel K block as a box of the grid: x-row segments, whole rows, planes, samples
     const int bx = n < 64 ? n : 64;
     const int by = 64 / bx < n ? 64 / bx : n;

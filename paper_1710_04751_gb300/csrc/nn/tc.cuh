@@ -204,6 +204,27 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     tmem_landed(v);
 }
 
+// Thread-block clusters: this CTA's rank, a barrier over all their threads (release / acquire),
+// the address of a shared-memory location in CTA `rank`, and a 16-byte store to it.
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_map(uint32_t saddr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void cluster_store4(uint32_t addr, float4 v) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z),
+                 "f"(v.w)
+                 : "memory");
+}
+
 // Shared-memory matrix descriptor of a K-major operand tile stored with the 128-byte
 // swizzle (rows of 64 BF16 = 128 bytes, groups of 8 rows 1024 bytes apart).  Fields:
 // start address >> 4 (bits 0-13), leading-dimension byte offset >> 4 (bits 16-29; not
