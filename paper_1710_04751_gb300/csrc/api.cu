@@ -178,6 +178,7 @@ DevParams<real> lbm::dev_params(const lbm_ctx* c) {
     p.e4_mode = P.e4_mode;
     p.adiabatic_mode = P.adiabatic_mode;
     p.boundary = P.boundary;
+    p.in_l2 = c->in_l2;
     p.nx = c->grid.nx;
     p.ny = c->grid.ny;
     p.nz = c->grid.nz;
@@ -275,6 +276,7 @@ int lbm::create_context(const lbm_grid* grid, int lattice, const lbm_params* par
     c->ncell = (int64_t)grid->nx * grid->ny * grid->nz;
     c->plane = plane_of(c->ncell);
     c->rsize = storage_bytes(o.precision);
+    c->in_l2 = state_fits_l2(copy_bytes(c));
     c->stream = (cudaStream_t)o.cuda_stream;
     c->cur = 0;
     c->steps = 0;

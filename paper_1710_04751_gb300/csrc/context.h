@@ -56,6 +56,8 @@ struct lbm_ctx {
     cudaStream_t capture = nullptr;
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
     bool graphs_failed = false;  // capture not possible here: launch the steps one by one
+    // state_fits_l2 of everything a step goes through: this context, the batch or all slabs
+    bool in_l2 = false;
     // (u_x, u_y, u_z, T) of lbm_init_fields in the arithmetic type, for its rounds of one step
     // and a reimposition; allocated at the first such call, freed with the context
     void* imposed = nullptr;
@@ -106,6 +108,9 @@ bool rounds_fused(lbm_ctx* c);
 // lbm_fields for cells [first, first + count): outs[w] (rho, ux, uy, uz, T; NULL = skip)
 // receive count values each.
 int fields_cells(lbm_ctx* c, double* const outs[5], int64_t first, int64_t count);
+
+// Bytes of one copy of a context's populations.
+inline int64_t copy_bytes(const lbm_ctx* c) { return (15 + c->Q) * c->plane * (int64_t)c->rsize; }
 
 // Bytes of the device arena of one context.
 size_t context_arena_bytes(const lbm_grid* g, int q, int precision);

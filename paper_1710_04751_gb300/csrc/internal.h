@@ -19,11 +19,20 @@ struct DevParams {
     real heat_source;   // uniform scalar source R (Eq. 4)
     real ext_fx, ext_fy, ext_fz;
     int e4_mode, adiabatic_mode, boundary;
+    int in_l2;          // a copy of the state stays in L2 from step to step (load_pop)
     int nx, ny, nz;
     int64_t ncell;      // nx * ny * nz
     int64_t plane;      // elements between population planes (ncell rounded up to 64)
     int64_t cell0;      // global index of cell 0 (slabs of a larger grid; 0 otherwise)
 };
+
+// Whether `bytes` of state, one copy of what a step works through, fit into the L2 cache next to
+// the copy being written, given that the loads let go of what they read (load_pop in
+// node.cuh).  Measured per step with / without, FP32: 72^3 D3Q15 (45 MB) 17.3 / 17.8 us, 80^3
+// (61 MB) 20.7 / 23.6, 91^3 D3Q7 (66 MB) 19.3 / 23.8, 88^3 (82 MB) 27.0 / 28.8, 100^3 D3Q7
+// (88 MB) 29.0 / 31.7, 92^3 (93 MB) 32.8 / 33.8; 96^3 (106 MB) 37.8 / 37.1, 128^3 (252 MB)
+// 81.2 / 78.6.  (GB300's L2 holds 128 MB.)
+inline bool state_fits_l2(int64_t bytes) { return bytes <= 96000000; }
 
 // Host-side view of one context's device buffers for the launchers.
 struct DevState {

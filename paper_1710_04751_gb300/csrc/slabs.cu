@@ -322,6 +322,9 @@ extern "C" int lbm_slabs_create(const lbm_grid* grid, int lattice, const lbm_par
         }
         s->m.push_back(c);
     }
+    int64_t copies = 0;  // a step goes through every slab
+    for (const lbm_ctx* c : s->m) copies += copy_bytes(c);
+    for (lbm_ctx* c : s->m) c->in_l2 = state_fits_l2(copies);
     // the streams and events of the fork / join (none for a single slab)
     for (int k = 0; k < nslabs && nslabs > 1; ++k) {
         cudaEvent_t e = nullptr;

@@ -104,9 +104,9 @@ __global__ void __launch_bounds__(128, (cavity_min_blocks<S, Q>() - (IMPOSE && c
     if (i >= p.nx) return;
     const bool interior = j >= 1 && j + 1 < p.ny && k >= 1 && k + 1 < p.nz;
     if (interior)
-        cavity_node<S, Q, true, UNIT, IMPOSE>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
+        cavity_node<S, Q, true, UNIT, IMPOSE, true>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
     else
-        cavity_node<S, Q, false, UNIT, IMPOSE>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
+        cavity_node<S, Q, false, UNIT, IMPOSE, true>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
 }
 
 // ---------------------------------------------------------------------------------
