@@ -149,8 +149,30 @@ __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15]
         dm.yy -= real(1.0 / 3.0);
         dm.zz -= real(1.0 / 3.0);
         const real inv_rho = real(1) / (real(1) + dm.m0);
-        UPow<real> u;
         Raw15<real> D;
+        if constexpr (!St::deviation && !IMPOSE) {
+            real ux, uy, uz;
+            flow_unit_nested<real>(dm, Fx, Fy, Fz, r, inv_rho, ux, uy, uz, D);
+            populations15_on<real>(D, p.wf[0], p.wf[1], p.wf[7], f);
+#pragma unroll
+            for (int a = 0; a < 15; ++a) Fout[a * P + c] = St::store(f[a], real(0));
+            if constexpr (Q == 15) {
+                thermal15_unit_nested<real>(T, m0, mx, my, mz, ux, uy, uz, r, D);
+                if constexpr (sizeof(real) == 8) {
+                    populations15_on<real>(D, p.wg[0] * T, p.wg[1] * T, p.wg[7] * T, g);
+#pragma unroll
+                    for (int a = 0; a < Q; ++a) Gout[a * P + c] = St::store(g[a], real(0));
+                    return;
+                }
+                populations15<real>(D, g);
+            } else {
+                thermal7_unit_nested<real>(T, m0, mx, my, mz, ux, uy, uz, r, g);
+            }
+#pragma unroll
+            for (int a = 0; a < Q; ++a) Gout[a * P + c] = St::store(fmad(p.wg[a], T, g[a]), real(0));
+            return;
+        }
+        UPow<real> u;
         real Ts = T;  // the stored state's temperature and velocity
         UPow<real> v;
         if constexpr (IMPOSE) {
