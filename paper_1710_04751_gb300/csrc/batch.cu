@@ -11,6 +11,7 @@
 #include "context.h"
 #include "lbm_batch.h"
 #include "node.cuh"
+#include "pdl.cuh"
 
 using namespace lbm;
 
@@ -133,6 +134,7 @@ __global__ void __launch_bounds__(THREADS, MINB)
     extern __shared__ __align__(16) unsigned char batch_smem[];
     __shared__ int next_tile;
     BatchMember<S>* cache = reinterpret_cast<BatchMember<S>*>(batch_smem);
+    pdl_begin();
     if (cache_all) block_copy(cache, members, (int)(count * sizeof(BatchMember<S>) / 4));
     if (threadIdx.x == 0) {
         if (blockIdx.x == 0) queue[parity ^ 1] = 0;
@@ -448,6 +450,17 @@ static int rebuild_tiles(lbm_batch* b) {
             n += member_tiles(b->members[m]->grid, m, b->tiling.threads * b->tiling.tile_factor,
                               b->tiling.mapping,
                               b->h_tiles + n);
+    // The last tiles a persistent grid takes set how long its slowest block is still at work when
+    // the others are done: as many as there are blocks go in pieces of one node per thread.
+    // (With the overlapped launches, 100 steps of 16 cavities: 20.55 -> 20.22 ms.)
+    const int64_t whole = n - std::min<int64_t>(n, (int64_t)b->sm_count * b->tiling.blocks_per_sm);
+    if (b->tiling.tile_factor > 1 && whole < n) {
+        std::vector<BatchTile> last(b->h_tiles + whole, b->h_tiles + n);
+        n = whole;
+        for (const BatchTile& t : last)
+            for (int c = 0; c < t.count; c += b->tiling.threads)
+                b->h_tiles[n++] = BatchTile{t.member, t.c0 + c, std::min(b->tiling.threads, t.count - c), 0};
+    }
     b->n_tiles = (int)n;
     *b->h_ntiles = (int)n;
     if (n > 0)
@@ -494,10 +507,10 @@ static cudaError_t launch_batch_step(const lbm_batch* b, int parity, cudaStream_
     const ParamsOf<S>* base;
     if constexpr (sizeof(typename Storage<S>::real) == 8) base = &b->params64[0];
     else base = &b->params32[0];
-    fn<<<b->grid, b->variant.threads, b->smem, st>>>(
-        static_cast<const BatchMember<S>*>(b->d_members), b->count, b->d_tiles, b->d_ntiles,
-        b->d_queue, b->cache_all, parity, *base);
-    return cudaGetLastError();
+    return launch_pdl_smem(fn, dim3((unsigned)b->grid), dim3((unsigned)b->variant.threads), b->smem, st,
+                           static_cast<const BatchMember<S>*>(b->d_members), b->count,
+                           (const BatchTile*)b->d_tiles, (const int*)b->d_ntiles, b->d_queue, b->cache_all, parity,
+                           *base);
 }
 
 template <typename S>
