@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(128, 1)
     __shared__ volatile int failed;
 
     if (*static_cast<volatile int*>(args.err) != 0) return;  // another CTA timed out
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * CBM, n0 = blockIdx.y * BN;
     const int nkb = 27 * args.chunks;
 
@@ -126,7 +126,8 @@ __global__ void __launch_bounds__(128, 1)
     const uint32_t tmem = *tmem_slot;
 
     int issued = 0;
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
+        const bool elected = elect_lane();
         // the tile's first voxel (its x0 is 0 unless a row holds several tiles)
         const int n = args.n;
         const int x0 = m0 % n, y0 = (m0 / n) % n, z0 = (m0 / (n * n)) % n, b0 = m0 / (n * n * n);
@@ -134,40 +135,43 @@ __global__ void __launch_bounds__(128, 1)
         for (int i = 0; i < nkb; ++i) {
             const int s = i % CSTAGES;
             const uint32_t ph = (uint32_t)(i / CSTAGES) & 1u;
-            if (i >= CSTAGES && !mbar_wait(empty + s, ph ^ 1u, args.err, 1, &failed)) {
+            if (i >= CSTAGES && !mbar_wait_warp(empty + s, ph ^ 1u, args.err, 1, &failed)) {
                 failed = 1;
                 break;
             }
-            if (failed) break;
             uint8_t* a = smem + s * L::STAGE;
             const int kz = tap / 9, ky = (tap / 3) % 3, kx = tap % 3;
-            mbar_expect_tx(full + s, L::STAGE);
-            tma_load_5d(a, &tmX, full + s, chunk * BKC, x0 + kx - 1, y0 + ky - 1, z0 + kz - 1, b0);
-            tma_load_2d(a + L::A_BYTES, &tmW, full + s, i * BKC, n0);
+            if (elected) {
+                mbar_expect_tx(full + s, L::STAGE);
+                tma_load_5d(a, &tmX, full + s, chunk * BKC, x0 + kx - 1, y0 + ky - 1, z0 + kz - 1, b0);
+                tma_load_2d(a + L::A_BYTES, &tmW, full + s, i * BKC, n0);
+            }
             ++issued;
             if (++chunk == args.chunks) {
                 chunk = 0;
                 ++tap;
             }
         }
-    } else if (warp == 1 && lane == 0) {
-        const uint32_t idesc = idesc_bf16_f32(CBM, BN);
+    } else if (warp == 1) {
+        const bool elected = elect_lane();
+        const uint32_t idesc = idesc_bf16_f32(CBM, BN), dhi = (uint32_t)(sdesc(0, BKC) >> 32);
         for (int i = 0; i < nkb; ++i) {
             const int s = i % CSTAGES;
             const uint32_t ph = (uint32_t)(i / CSTAGES) & 1u;
-            if (failed || !mbar_wait(full + s, ph, args.err, 2, &failed)) {
+            if (!mbar_wait_warp(full + s, ph, args.err, 2, &failed)) {
                 failed = 1;
                 break;
             }
             tc_fence_after();
-            const uint32_t a = smem_u32(smem + s * L::STAGE), b = a + L::A_BYTES;
+            const uint32_t a = (uint32_t)sdesc(smem_u32(smem + s * L::STAGE), BKC), b = a + (L::A_BYTES >> 4);
+            if (elected) {
 #pragma unroll
-            for (int kk = 0; kk < BKC / 16; ++kk)
-                mma_bf16(tmem, sdesc(a + kk * 32, BKC), sdesc(b + kk * 32, BKC), idesc,
-                         (i > 0 || kk > 0) ? 1u : 0u);
-            mma_commit(empty + s);
+                for (int kk = 0; kk < BKC / 16; ++kk)
+                    mma_bf16(tmem, a + kk * 2, dhi, b + kk * 2, dhi, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+                mma_commit(empty + s);
+            }
         }
-        mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
+        if (elected) mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
     }
     __syncwarp();
     if (!mbar_wait(done, 0, args.err, 3)) failed = 1;
@@ -309,7 +313,7 @@ __global__ void __launch_bounds__(128, 1)
                     const uint32_t at = alo + (uint32_t)(t * (CBM * 64 >> 4)) + (uint32_t)ky * window;
 #pragma unroll
                     for (int kk = 0; kk < 2; ++kk)
-                        mma_bf16_halves(tmem + (uint32_t)(t * W), at + kk * 2, dhi,
+                        mma_bf16(tmem + (uint32_t)(t * W), at + kk * 2, dhi,
                                         blo + (uint32_t)(ky * (3 * B_TILE >> 4)) + kk * 2, dhi, idesc,
                                         (i > 0 || ky > 0 || kk > 0) ? 1u : 0u);
                 }
@@ -486,7 +490,7 @@ __global__ void __launch_bounds__(128, 1)
     __shared__ volatile int failed;
 
     if (*static_cast<volatile int*>(args.err) != 0) return;  // another CTA timed out
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * CBM, n0 = blockIdx.y * BN;
     const int kb0 = blockIdx.z * args.kb_per_split;
     const int nkb = min(args.kb_per_split, args.kblocks - kb0);
@@ -507,7 +511,8 @@ __global__ void __launch_bounds__(128, 1)
     const uint32_t tmem = *tmem_slot;
 
     int issued = 0;
-    if (nkb > 0 && warp == 0 && lane == 0) {
+    if (nkb > 0 && warp == 0) {
+        const bool elected = elect_lane();
         const int ln = args.ln, mask = (1 << ln) - 1;
         // the (tap, channel) groups of the M tile do not change along K
         int gx[4], gy[4], gz[4], gc[4];
@@ -526,44 +531,50 @@ __global__ void __launch_bounds__(128, 1)
         for (int i = 0; i < nkb; ++i) {
             const int s = i % WG_STAGES;
             const uint32_t ph = (uint32_t)(i / WG_STAGES) & 1u;
-            if (i >= WG_STAGES && !mbar_wait(empty + s, ph ^ 1u, args.err, 1, &failed)) {
+            if (i >= WG_STAGES && !mbar_wait_warp(empty + s, ph ^ 1u, args.err, 1, &failed)) {
                 failed = 1;
                 break;
             }
-            if (failed) break;
             uint8_t* a = smem + s * L::STAGE;
-            mbar_expect_tx(full + s, L::STAGE);
             const int v0 = (kb0 + i) << 6;
             const int x0 = v0 & mask, y0 = (v0 >> ln) & mask, z0 = (v0 >> (2 * ln)) & mask, b0 = v0 >> (3 * ln);
+            if (elected) {
+                mbar_expect_tx(full + s, L::STAGE);
 #pragma unroll
-            for (int g = 0; g < 4; ++g)
-                tma_load_5d(a + g * 4096, &tmX, full + s, gc[g], x0 + gx[g], y0 + gy[g], z0 + gz[g], b0);
+                for (int g = 0; g < 4; ++g)
+                    tma_load_5d(a + g * 4096, &tmX, full + s, gc[g], x0 + gx[g], y0 + gy[g], z0 + gz[g], b0);
 #pragma unroll
-            for (int j = 0; j < BN / L::BB; ++j)
-                tma_load_2d(a + L::A_BYTES + j * L::B_GROUP, &tmB, full + s, n0 + j * L::BB, v0);
+                for (int j = 0; j < BN / L::BB; ++j)
+                    tma_load_2d(a + L::A_BYTES + j * L::B_GROUP, &tmB, full + s, n0 + j * L::BB, v0);
+            }
             ++issued;
         }
-    } else if (nkb > 0 && warp == 1 && lane == 0) {
+    } else if (nkb > 0 && warp == 1) {
+        const bool elected = elect_lane();
         const uint32_t idesc = idesc_bf16_f32_mn(CBM, BN);
         // with one B box the leading offset is never used: give it the K stride too
         constexpr uint32_t b_lbo = BN / L::BB > 1 ? L::B_GROUP : L::B_ATOM;
         for (int i = 0; i < nkb; ++i) {
             const int s = i % WG_STAGES;
             const uint32_t ph = (uint32_t)(i / WG_STAGES) & 1u;
-            if (failed || !mbar_wait(full + s, ph, args.err, 2, &failed)) {
+            if (!mbar_wait_warp(full + s, ph, args.err, 2, &failed)) {
                 failed = 1;
                 break;
             }
             tc_fence_after();
-            const uint32_t a = smem_u32(smem + s * L::STAGE), b = a + L::A_BYTES;
+            const uint32_t a = smem_u32(smem + s * L::STAGE);
+            const uint64_t ad = sdesc_mn(a, 4096, 512, 4);
+            const uint64_t bd = sdesc_mn(a + L::A_BYTES, b_lbo, L::B_ATOM, L::B_LAYOUT);
+            if (elected) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)  // K = 16 per MMA: two atoms of 8 K rows
-                mma_bf16(tmem, sdesc_mn(a + kk * 1024, 4096, 512, 4),
-                         sdesc_mn(b + kk * 2 * L::B_ATOM, b_lbo, L::B_ATOM, L::B_LAYOUT), idesc,
-                         (i > 0 || kk > 0) ? 1u : 0u);
-            mma_commit(empty + s);
+                for (int kk = 0; kk < 4; ++kk)  // K = 16 per MMA: two atoms of 8 K rows
+                    mma_bf16(tmem, (uint32_t)ad + kk * 64, (uint32_t)(ad >> 32),
+                                    (uint32_t)bd + kk * (2 * L::B_ATOM >> 4), (uint32_t)(bd >> 32), idesc,
+                                    (i > 0 || kk > 0) ? 1u : 0u);
+                mma_commit(empty + s);
+            }
         }
-        mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
+        if (elected) mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
     }
     __syncwarp();
     if (nkb > 0 && !mbar_wait(done, 0, args.err, 3)) failed = 1;
@@ -765,7 +776,7 @@ __global__ void __launch_bounds__(128, 1)
                         // dZ row y0 + row - (ky - 1): place d = row - ky of this slot, or of one before
                         const int back = row >= ky ? 0 : (ky - row + RB - 1) / RB;
                         const int d = row - ky + back * RB;
-                        mma_bf16_halves(tmem + (uint32_t)(ky * W9_N), a + kk * 64, ahi,
+                        mma_bf16(tmem + (uint32_t)(ky * W9_N), a + kk * 64, ahi,
                                         z[back] + (uint32_t)(((d - row) * line + kk * 1024) >> 4), ahi, idesc, acc);
                     }
                     acc = 1;

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(128, 1)
 
     // a CTA that starts after another one timed out does nothing
     if (*static_cast<volatile int*>(args.err) != 0) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     const int m0 = blockIdx.x * BM * MT, n0 = blockIdx.y * BN;
     const int kb_total = (args.K + BK - 1) / BK;
     const int kb0 = blockIdx.z * args.kblocks_per_split;
@@ -89,43 +89,48 @@ __global__ void __launch_bounds__(128, 1)
     const uint32_t tmem = *tmem_slot;
 
     int issued = 0;  // producer: stages loaded
-    if (nkb > 0 && warp == 0 && lane == 0 && !args.withhold_loads) {
+    if (nkb > 0 && warp == 0 && !args.withhold_loads) {
+        const bool elected = elect_lane();
         for (int i = 0; i < nkb; ++i) {
             const int s = i % STAGES;
             const uint32_t ph = (uint32_t)(i / STAGES) & 1u;
-            if (i >= STAGES && !mbar_wait(empty + s, ph ^ 1u, args.err, 1, &failed, args.wait_ns)) {
+            if (i >= STAGES && !mbar_wait_warp(empty + s, ph ^ 1u, args.err, 1, &failed, args.wait_ns)) {
                 failed = 1;
                 break;
             }
-            if (failed) break;
             uint8_t* a = smem + s * L::STAGE;
-            mbar_expect_tx(full + s, L::STAGE);
+            if (elected) {
+                mbar_expect_tx(full + s, L::STAGE);
 #pragma unroll
-            for (int t = 0; t < MT; ++t)
-                tma_load_2d(a + t * L::A_BYTES, &tmA, full + s, (kb0 + i) * BK, m0 + t * BM);
-            tma_load_2d(a + MT * L::A_BYTES, &tmB, full + s, (kb0 + i) * BK, n0);
+                for (int t = 0; t < MT; ++t)
+                    tma_load_2d(a + t * L::A_BYTES, &tmA, full + s, (kb0 + i) * BK, m0 + t * BM);
+                tma_load_2d(a + MT * L::A_BYTES, &tmB, full + s, (kb0 + i) * BK, n0);
+            }
             ++issued;
         }
-    } else if (nkb > 0 && warp == 1 && lane == 0) {
-        const uint32_t idesc = idesc_bf16_f32(BM, BN);
+    } else if (nkb > 0 && warp == 1) {
+        const bool elected = elect_lane();
+        const uint32_t idesc = idesc_bf16_f32(BM, BN), dhi = (uint32_t)(sdesc_k_sw128(0) >> 32);
         for (int i = 0; i < nkb; ++i) {
             const int s = i % STAGES;
             const uint32_t ph = (uint32_t)(i / STAGES) & 1u;
-            if (failed || !mbar_wait(full + s, ph, args.err, 2, &failed, args.wait_ns)) {
+            if (!mbar_wait_warp(full + s, ph, args.err, 2, &failed, args.wait_ns)) {
                 failed = 1;
                 break;
             }
             tc_fence_after();
-            const uint32_t a = smem_u32(smem + s * L::STAGE), b = a + MT * L::A_BYTES;
+            const uint32_t a = (uint32_t)sdesc_k_sw128(smem_u32(smem + s * L::STAGE)), b = a + (MT * L::A_BYTES >> 4);
+            if (elected) {
 #pragma unroll
-            for (int t = 0; t < MT; ++t)
+                for (int t = 0; t < MT; ++t)
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                    mma_bf16(tmem + (uint32_t)(t * BN), sdesc_k_sw128(a + t * L::A_BYTES + kk * 32),
-                             sdesc_k_sw128(b + kk * 32), idesc, (i > 0 || kk > 0) ? 1u : 0u);
-            mma_commit(empty + s);
+                    for (int kk = 0; kk < BK / 16; ++kk)
+                        mma_bf16(tmem + (uint32_t)(t * BN), a + (uint32_t)(t * L::A_BYTES >> 4) + kk * 2, dhi,
+                                 b + kk * 2, dhi, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+                mma_commit(empty + s);
+            }
         }
-        mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
+        if (elected) mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
     }
     __syncwarp();
     // the accumulator is complete (or the MMA thread gave up) once `done` fires

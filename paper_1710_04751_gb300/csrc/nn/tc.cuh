@@ -96,8 +96,8 @@ __device__ __forceinline__ bool elect_lane() {
 }
 // mbar_wait by a whole warp: every lane's answer is the same.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* err, int code,
-                                               const volatile int* abort) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code, abort));
+                                               const volatile int* abort, uint64_t limit_ns = 2000000000ull) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, err, code, abort, limit_ns));
 }
 
 // 2D tiled TMA load of the box at (c0 = innermost element, c1 = row) into shared memory,
@@ -144,23 +144,13 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
                  : "memory");
 }
 
-// D (TMEM) (+)= A (smem, descriptor) * B (smem, descriptor)^T; one thread issues.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
+// D (TMEM) (+)= A (smem, descriptor) * B (smem, descriptor)^T; one thread issues.  Each
+// descriptor comes in two halves: the upper one (strides and layout) does not change over an
+// operand, and the lower one moves by an address step >> 4, so that the issuing thread spends an
+// addition per operand and MMA.  (A thread that builds 64-bit descriptors from runtime strides
+// for every MMA takes longer than a narrow MMA does.)
+__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
                                          uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The same with each descriptor in two halves: the upper one (strides and layout) does not change
-// over an operand, and the lower one moves by an address step >> 4, so that the issuing thread
-// spends an addition per operand and MMA.  (A thread that builds 64-bit descriptors from
-// runtime strides for every MMA takes longer than a narrow MMA does.)
-__device__ __forceinline__ void mma_bf16_halves(uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
-                                                uint32_t bhi, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
         "setp.ne.b32 p, %6, 0;\n\t"
