@@ -59,7 +59,7 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, int bkc) {
 __device__ __forceinline__ void conv_store16(void* out, int N, int mode, const float* __restrict__ bias,
                                              int row, int col0, float (&v)[16]) {
     if (col0 >= N) return;
-    const bool whole = col0 + 16 <= N && (N % 8) == 0;  // 16-byte stores
+    const bool whole = (N % 8) == 0;  // 16-byte stores of 8 (BF16) or 4 columns: none is cut
     if (mode == CONV_BIAS_RELU_BF16) {
         __nv_bfloat16* C = static_cast<__nv_bfloat16*>(out) + (int64_t)row * N;
 #pragma unroll
@@ -70,7 +70,7 @@ __device__ __forceinline__ void conv_store16(void* out, int N, int mode, const f
 #pragma unroll
             for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
             reinterpret_cast<uint4*>(C + col0)[0] = pk[0];
-            reinterpret_cast<uint4*>(C + col0)[1] = pk[1];
+            if (col0 + 8 < N) reinterpret_cast<uint4*>(C + col0)[1] = pk[1];
         } else {
 #pragma unroll
             for (int j = 0; j < 16; ++j)
@@ -81,8 +81,9 @@ __device__ __forceinline__ void conv_store16(void* out, int N, int mode, const f
         if (whole) {
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                reinterpret_cast<float4*>(C + col0)[j] =
-                    make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                if (col0 + 4 * j < N)
+                    reinterpret_cast<float4*>(C + col0)[j] =
+                        make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         } else {
 #pragma unroll
             for (int j = 0; j < 16; ++j)
@@ -214,20 +215,40 @@ __global__ void __launch_bounds__(128, 1)
 // ---------------------------------------------------------------------------------
 struct X3Args {
     int N, n, chunks, cin;  // chunks of 32 input channels
-    int ntiles;             // tiles of BN output channels
-    int by, mt;             // rows per 128-voxel tile, tiles per CTA
+    int ntiles, items;      // tiles of BN output channels; (group of MT tiles, channel tile) pairs
+    int by, mt;             // rows per 128-voxel tile, tiles per item
     int a_bytes;            // one stage's input box: (mt by + 2) n 64 bytes
     int stage_bytes;        // a_bytes + 9 BN 64
     int stages;
-    uint32_t tmem_cols;     // mt 3 BN rounded up to a power of two
     int mode;
     void* C;
     const float* bias;
     int* err;
 };
+constexpr int kX3Threads = 320;  // producer, MMA, two sets of four epilogue warps
 
+// One item's place: first row, grid position, output channels, the kz planes inside the grid.
+struct X3Item {
+    int m0, n0, y0, z0, b0, kz0, kz1;
+    __device__ X3Item(const X3Args& a, int item, int bn) {
+        const int mg = item / a.ntiles, n = a.n;
+        n0 = (item - mg * a.ntiles) * bn;
+        m0 = mg * a.mt * CBM;
+        y0 = (m0 / n) % n, z0 = (m0 / (n * n)) % n, b0 = m0 / (n * n * n);
+        kz0 = z0 == 0 ? 1 : 0, kz1 = z0 == n - 1 ? 2 : 3;
+    }
+};
+
+// Persistent: a CTA per SM takes items by stride.  The producer warp keeps the stage ring full
+// across items, the MMA warp fills one of two accumulator sets while the epilogue warps drain
+// the other.  (With a CTA per item, two on an SM, the 64^3 96 -> 32 layer, batch 2, spent 25 of
+// 87 us in 2048 CTAs' set-up and 22 in epilogues.)  Per call with the host wait, that form / this
+// one: that layer 110 / 92 us, 64^3 32 -> 32 77 / 64, 32^3 64 -> 192 in FP32 80 / 68, 128^3
+// 32 -> 32 234 / 169, 16^3 128 -> 128 (an item per CTA) 35 / 35.  The tensor pipe is then 70% busy
+// with operand reads (67 cycles per MMA of 96 columns); sharing the weights in clusters of two
+// by TMA multicast was no faster.
 template <int BN>
-__global__ void __launch_bounds__(128, 1)
+__global__ void __launch_bounds__(kX3Threads, 1)
     conv_x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
                    X3Args args) {
     extern __shared__ uint8_t x3_smem_raw[];
@@ -236,20 +257,17 @@ __global__ void __launch_bounds__(128, 1)
     const int S = args.stages;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * args.stage_bytes);
     uint64_t* empty = full + S;
-    uint64_t* done = empty + S;
+    uint64_t* acc_full = empty + S;   // [2]
+    uint64_t* acc_empty = acc_full + 2;
+    uint64_t* done = acc_empty + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     __shared__ volatile int failed;
-    __shared__ float edge[2][4][2][16];  // P_0 of a warp's last row, P_2 of its first
+    __shared__ float edge[2][2][4][2][16];  // of each epilogue set: P_0 of a warp's last row, P_2 of its first
     constexpr int W = 3 * BN, B_TILE = BN * 64;
 
     if (*static_cast<volatile int*>(args.err) != 0) return;  // another CTA timed out
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int MT = args.mt, n = args.n;
-    const int mg = blockIdx.x / args.ntiles, n0 = (blockIdx.x - mg * args.ntiles) * BN;
-    const int m0 = mg * MT * CBM;
-    const int y0 = (m0 / n) % n, z0 = (m0 / (n * n)) % n, b0 = m0 / (n * n * n);
-    const int kz0 = z0 == 0 ? 1 : 0, kz1 = z0 == n - 1 ? 2 : 3;  // planes inside the grid
-    const int nkb = (kz1 - kz0) * args.chunks;                   // stages: (kz, chunk)
 
     if (threadIdx.x == 0) {
         failed = 0;
@@ -257,10 +275,14 @@ __global__ void __launch_bounds__(128, 1)
             mbar_init(full + s, 1);
             mbar_init(empty + s, 1);
         }
+        for (int s = 0; s < 2; ++s) {
+            mbar_init(acc_full + s, 1);
+            mbar_init(acc_empty + s, 8);  // a lane of every epilogue warp
+        }
         mbar_init(done, 1);
         mbar_fence_init();
     }
-    if (warp == 0) tmem_alloc(tmem_slot, args.tmem_cols);
+    if (warp == 0) tmem_alloc(tmem_slot, 512);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -269,112 +291,144 @@ __global__ void __launch_bounds__(128, 1)
     int issued = 0;
     if (warp == 0) {
         const bool elected = elect_lane();
-        int kz = kz0, chunk = 0, s = 0;
+        int s = 0;
         uint32_t ph = 1;  // parity of the slot's last release
-        for (int i = 0; i < nkb; ++i) {
-            if (i >= S && !mbar_wait_warp(empty + s, ph, args.err, 1, &failed)) {
-                failed = 1;
-                break;
-            }
-            uint8_t* a = smem + s * args.stage_bytes;
-            if (elected) {
-                mbar_expect_tx(full + s, (uint32_t)(args.a_bytes + 9 * B_TILE));
-                tma_load_5d(a, &tmX, full + s, chunk * 32, 0, y0 - 1, z0 + kz - 1, b0);
+        bool ok = true;
+        for (int item = blockIdx.x; ok && item < args.items; item += gridDim.x) {
+            const X3Item it(args, item, BN);
+            for (int kz = it.kz0; ok && kz < it.kz1; ++kz)
+                for (int chunk = 0; chunk < args.chunks; ++chunk) {
+                    if (issued >= S && !mbar_wait_warp(empty + s, ph, args.err, 1, &failed)) {
+                        failed = 1;
+                        ok = false;
+                        break;
+                    }
+                    uint8_t* a = smem + s * args.stage_bytes;
+                    if (elected) {
+                        mbar_expect_tx(full + s, (uint32_t)(args.a_bytes + 9 * B_TILE));
+                        tma_load_5d(a, &tmX, full + s, chunk * 32, 0, it.y0 - 1, it.z0 + kz - 1, it.b0);
 #pragma unroll
-                for (int t = 0; t < 9; ++t)  // (ky, kx) of this kz
-                    tma_load_2d(a + args.a_bytes + t * B_TILE, &tmW, full + s,
-                                (kz * 9 + t) * args.cin + chunk * 32, n0);
-            }
-            ++issued;
-            if (++s == S) s = 0, ph ^= 1u;
-            if (++chunk == args.chunks) {
-                chunk = 0;
-                ++kz;
-            }
+                        for (int t = 0; t < 9; ++t)  // (ky, kx) of this kz
+                            tma_load_2d(a + args.a_bytes + t * B_TILE, &tmW, full + s,
+                                        (kz * 9 + t) * args.cin + chunk * 32, it.n0);
+                    }
+                    ++issued;
+                    if (++s == S) s = 0, ph ^= 1u;
+                }
         }
     } else if (warp == 1) {
         const bool elected = elect_lane();
         const uint32_t idesc = idesc_bf16_f32(CBM, W), dhi = (uint32_t)(sdesc_k_sw64(0) >> 32);
         const uint32_t window = (uint32_t)(n * 64 >> 4);
-        int s = 0;
+        int s = 0, k = 0;
         uint32_t ph = 0;
-        for (int i = 0; i < nkb; ++i) {
-            if (!mbar_wait_warp(full + s, ph, args.err, 2, &failed)) {
+        bool ok = true;
+        for (int item = blockIdx.x; ok && item < args.items; item += gridDim.x, ++k) {
+            const X3Item it(args, item, BN);
+            const uint32_t acc = tmem + (uint32_t)((k & 1) * 256);
+            if (k >= 2 && !mbar_wait_warp(acc_empty + (k & 1), (uint32_t)(k / 2 + 1) & 1u, args.err, 5, &failed)) {
+                failed = 1;
+                break;
+            }
+            const int nkb = (it.kz1 - it.kz0) * args.chunks;
+            for (int i = 0; i < nkb; ++i) {
+                if (!mbar_wait_warp(full + s, ph, args.err, 2, &failed)) {
+                    failed = 1;
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t stage = smem_u32(smem + s * args.stage_bytes);
+                const uint32_t alo = (uint32_t)sdesc_k_sw64(stage);
+                const uint32_t blo = (uint32_t)sdesc_k_sw64(stage + (uint32_t)args.a_bytes);
+                if (elected) {
+                    for (int t = 0; t < MT; ++t) {
+#pragma unroll
+                        for (int ky = 0; ky < 3; ++ky) {  // the window of tap ky: 128 t + n ky rows of 64 bytes on
+                            const uint32_t at = alo + (uint32_t)(t * (CBM * 64 >> 4)) + (uint32_t)ky * window;
+                            const uint32_t bt = blo + (uint32_t)(ky * (3 * B_TILE >> 4));
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk)
+                                mma_bf16(acc + (uint32_t)(t * W), at + kk * 2, dhi, bt + kk * 2, dhi, idesc,
+                                         (i > 0 || ky > 0 || kk > 0) ? 1u : 0u);
+                        }
+                    }
+                    mma_commit(empty + s);
+                }
+                if (++s == S) s = 0, ph ^= 1u;
+            }
+            if (elected && ok) mma_commit(acc_full + (k & 1));
+        }
+        if (elected) mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
+    } else {
+        const int quarter = warp & 3, set = (warp - 2) >> 2;  // a warp reads the TMEM lanes of its index mod 4
+        const int x = (quarter * 32 + lane) & (n - 1);
+        const bool first = x == 0, last = x == n - 1;
+        int k = 0, par = 0;
+        for (int item = blockIdx.x; item < args.items; item += gridDim.x, ++k) {
+            const X3Item it(args, item, BN);
+            // the four warps of a set give up together: they meet at its barrier below
+            const bool there = mbar_wait_warp(acc_full + (k & 1), (uint32_t)(k / 2) & 1u, args.err, 3, &failed);
+            if (!bar_all(1 + set, 128, there)) {
                 failed = 1;
                 break;
             }
             tc_fence_after();
-            const uint32_t alo = (uint32_t)sdesc_k_sw64(smem_u32(smem + s * args.stage_bytes));
-            const uint32_t blo = (uint32_t)sdesc_k_sw64(smem_u32(smem + s * args.stage_bytes) + args.a_bytes);
-            if (elected) {
-              for (int t = 0; t < MT; ++t) {
-#pragma unroll
-                for (int ky = 0; ky < 3; ++ky) {  // the window of tap ky: t 128 + ky n rows of 64 bytes on
-                    const uint32_t at = alo + (uint32_t)(t * (CBM * 64 >> 4)) + (uint32_t)ky * window;
-#pragma unroll
-                    for (int kk = 0; kk < 2; ++kk)
-                        mma_bf16(tmem + (uint32_t)(t * W), at + kk * 2, dhi,
-                                        blo + (uint32_t)(ky * (3 * B_TILE >> 4)) + kk * 2, dhi, idesc,
-                                        (i > 0 || ky > 0 || kk > 0) ? 1u : 0u);
-                }
-              }
-              mma_commit(empty + s);
-            }
-            if (++s == S) s = 0, ph ^= 1u;
-        }
-        if (elected) mma_commit(done);  // also when stopped early: every issued MMA drains before dealloc
-    }
-    __syncwarp();
-    if (!mbar_wait(done, 0, args.err, 3)) failed = 1;
-    __syncthreads();
-    const bool ok = !failed;
-    if (warp == 0 && lane == 0 && failed) {  // let every started copy land
-        for (int i = max(0, issued - S); i < issued; ++i)
-            mbar_wait(full + (i % S), (uint32_t)(i / S) & 1u, args.err, 4);
-    }
-    tc_fence_after();
-    if (ok) {
-        const int x = (warp * 32 + lane) & (n - 1);
-        const bool first = x == 0, last = x == n - 1;
-        int par = 0;
-        for (int t = 0; t < MT; ++t) {
-            const int row = m0 + t * CBM + warp * 32 + lane;
-            const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * W);
-#pragma unroll 1
-            for (int c = 0; c < BN; c += 16, par ^= 1) {
+            const uint32_t acc = tmem + (uint32_t)((k & 1) * 256) + ((uint32_t)(quarter * 32) << 16);
+            // the item's MT BN / 16 chunks of 16 channels go to the two sets in turn
+            for (int q = set; q < MT * (BN / 16); q += 2, par ^= 1) {
+                const int t = q / (BN / 16), c = (q - t * (BN / 16)) * 16;
+                const uint32_t base = acc + (uint32_t)(t * W + c);
                 float p0[16], v[16], p2[16];
-                tmem_ld16_issue(base + (uint32_t)c, p0);
-                tmem_ld16_issue(base + (uint32_t)(BN + c), v);
-                tmem_ld16_issue(base + (uint32_t)(2 * BN + c), p2);
+                tmem_ld16_issue(base, p0);
+                tmem_ld16_issue(base + (uint32_t)BN, v);
+                tmem_ld16_issue(base + (uint32_t)(2 * BN), p2);
                 tmem_wait_ld();
                 tmem_landed(p0);
                 tmem_landed(v);
                 tmem_landed(p2);
                 if (n > 32) {  // block-uniform
+                    float(&e)[4][2][16] = edge[set][par];
                     if (lane == 31) {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) edge[par][warp][0][j] = p0[j];
+                        for (int j = 0; j < 16; ++j) e[quarter][0][j] = p0[j];
                     }
                     if (lane == 0) {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) edge[par][warp][1][j] = p2[j];
+                        for (int j = 0; j < 16; ++j) e[quarter][1][j] = p2[j];
                     }
-                    __syncthreads();
-                }
+                    bar_sync(1 + set, 128);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    float l = __shfl_up_sync(0xffffffffu, p0[j], 1), r = __shfl_down_sync(0xffffffffu, p2[j], 1);
-                    if (lane == 0 && !first) l = edge[par][warp - 1][0][j];
-                    if (lane == 31 && !last) r = edge[par][warp + 1][1][j];
-                    v[j] += (first ? 0.f : l) + (last ? 0.f : r);
+                    for (int j = 0; j < 16; ++j) {
+                        float l = __shfl_up_sync(0xffffffffu, p0[j], 1), r = __shfl_down_sync(0xffffffffu, p2[j], 1);
+                        if (lane == 0 && !first) l = e[quarter - 1][0][j];
+                        if (lane == 31 && !last) r = e[quarter + 1][1][j];
+                        v[j] += (first ? 0.f : l) + (last ? 0.f : r);
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const float l = __shfl_up_sync(0xffffffffu, p0[j], 1);
+                        const float r = __shfl_down_sync(0xffffffffu, p2[j], 1);
+                        v[j] += (first ? 0.f : l) + (last ? 0.f : r);
+                    }
                 }
-                conv_store16(args.C, args.N, args.mode, args.bias, row, n0 + c, v);
+                conv_store16(args.C, args.N, args.mode, args.bias, it.m0 + t * CBM + quarter * 32 + lane, it.n0 + c, v);
             }
+            tc_fence_before();
+            if (lane == 0) mbar_arrive(acc_empty + (k & 1));
         }
+    }
+    __syncwarp();
+    if (!mbar_wait(done, 0, args.err, 3)) failed = 1;
+    if (warp == 0 && lane == 0 && failed) {  // let every started copy land
+        for (int i = max(0, issued - S); i < issued; ++i)
+            mbar_wait(full + (i % S), (uint32_t)(i / S) & 1u, args.err, 4);
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, args.tmem_cols);
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -872,21 +926,20 @@ cudaError_t launch_conv(const CUtensorMap& tx, const CUtensorMap& tw, const Conv
     return cudaGetLastError();
 }
 
-constexpr int kX3Smem = 104 * 1024;     // stages of one of two CTAs on an SM
-constexpr int kX3SmemMax = 200 * 1024;  // of one alone
+constexpr int kX3Smem = 216 * 1024;  // stages of a CTA
 constexpr int kSMs = 152;
 
 template <int BN>
-cudaError_t launch_x3(const CUtensorMap& tx, const CUtensorMap& tw, const X3Args& a, int groups, cudaStream_t st) {
+cudaError_t launch_x3(const CUtensorMap& tx, const CUtensorMap& tw, const X3Args& a, cudaStream_t st) {
     static std::once_flag once;
     static cudaError_t attr = cudaSuccess;
     std::call_once(once, [] {
         attr = cudaFuncSetAttribute(conv_x3_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    1024 + kX3SmemMax + 256);
+                                    1024 + kX3Smem + 256);
     });
     if (attr != cudaSuccess) return attr;
-    const size_t smem = 1024 + (size_t)a.stages * a.stage_bytes + 256;
-    conv_x3_kernel<BN><<<groups * a.ntiles, 128, smem, st>>>(tx, tw, a);
+    // the whole budget whatever the stages take: one CTA per SM owns the tensor memory
+    conv_x3_kernel<BN><<<std::min(a.items, kSMs), kX3Threads, 1024 + kX3Smem + 256, st>>>(tx, tw, a);
     return cudaGetLastError();
 }
 
@@ -945,31 +998,24 @@ cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const _
         const int by1 = 128 / n, b_bytes = 9 * bn * 64;
         const int64_t tiles = (int64_t)B * n * n * n / CBM;
         auto stage_of = [&](int mt) { return (mt * by1 + 2) * n * 64 + b_bytes; };
-        // Two CTAs per SM, so that one computes while the other drains its accumulators: two
-        // stages in kX3Smem and at most half of the tensor memory each; within that the most
-        // tiles per CTA (they share the weights and the halo rows) that leave every SM a CTA.
-        // 64^3, batch 2, 96 -> 32 channels: 2 tiles 129 us a call, 1 tile 166, 4 tiles and one
-        // CTA per SM 153.
+        // as many tiles per item as two sets of accumulators of 256 columns and four stages allow
+        // (they share the weights and the halo rows), and as leave every SM an item
         int mt = 4;
-        while (mt > 1 && (mt * 3 * bn > 256 || mt * by1 > n || 2 * stage_of(mt) > kX3Smem ||
+        while (mt > 1 && (mt * 3 * bn > 256 || mt * by1 > n || 4 * stage_of(mt) > kX3Smem ||
                           tiles / mt * ntiles < kSMs))
             mt >>= 1;
         const int stage = stage_of(mt);
-        const int stages = std::min(4, std::max(kX3Smem, kX3SmemMax * (2 * stage > kX3Smem)) / stage);
-        uint32_t cols = 32;
-        while ((int)cols < mt * 3 * bn) cols <<= 1;
         CUtensorMap tx, tw;
         if (!make_x_map(&tx, X, B, n, cin, 32, n, mt * by1 + 2, 1, 1) ||
             !make_w_map(&tw, W, cout, 27 * cin, ldw, 32, bn))
             return cudaErrorInvalidValue;
-        X3Args a{cout, n, cin / 32, cin, ntiles, by1, mt, (mt * by1 + 2) * n * 64, stage, stages, cols,
-                 mode, out, bias, err};
-        const int groups = (int)(tiles / mt);
+        X3Args a{cout, n, cin / 32, cin, ntiles, (int)(tiles / mt) * ntiles, by1, mt, (mt * by1 + 2) * n * 64, stage,
+                 std::min(8, kX3Smem / stage), mode, out, bias, err};
         switch (bn) {
-        case 16: return launch_x3<16>(tx, tw, a, groups, st);
-        case 32: return launch_x3<32>(tx, tw, a, groups, st);
-        case 48: return launch_x3<48>(tx, tw, a, groups, st);
-        default: return launch_x3<64>(tx, tw, a, groups, st);
+        case 16: return launch_x3<16>(tx, tw, a, st);
+        case 32: return launch_x3<32>(tx, tw, a, st);
+        case 48: return launch_x3<48>(tx, tw, a, st);
+        default: return launch_x3<64>(tx, tw, a, st);
         }
     }
     CUtensorMap tx, tw;
