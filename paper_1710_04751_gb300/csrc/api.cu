@@ -5,6 +5,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <chrono>
 #include <new>
 #include <string>
@@ -355,48 +356,84 @@ extern "C" int lbm_create(const lbm_grid* grid, int lattice, double Ra, double P
     return lbm_create_params(grid, lattice, &p, opt, out);
 }
 
-// One step (and, when the step count reaches a multiple of the residual interval, the
-// residual check) launched on stream `st` from buffer `cur`.
+// The residual check of the state in buffer `cur`, if the step count has reached a multiple of the
+// residual interval.
 template <typename S>
-static cudaError_t enqueue_step(lbm_ctx* c, const ParamsOf<S>& p, int cur, int64_t steps_after,
-                                cudaStream_t st) {
-    cudaError_t e = launch_step<S>(c->dev, cur, p, st);
+static cudaError_t enqueue_check(lbm_ctx* c, const ParamsOf<S>& p, int cur, int64_t steps_after,
+                                 cudaStream_t st) {
     const int R = c->opt.residual_interval;
-    if (e == cudaSuccess && R > 0 && steps_after % R == 0) {
-        e = cudaMemsetAsync(c->dev.resid_bits, 0, sizeof(unsigned long long), st);
-        if (e == cudaSuccess) e = launch_residual<S>(c->dev, cur ^ 1, p, 1, st);
-    }
-    return e;
+    if (R <= 0 || steps_after % R != 0) return cudaSuccess;
+    const cudaError_t e = cudaMemsetAsync(c->dev.resid_bits, 0, sizeof(unsigned long long), st);
+    return e != cudaSuccess ? e : launch_residual<S>(c->dev, cur, p, 1, st);
 }
 
-// The graph of residual_interval steps starting from buffer `cur` (captured on first use;
-// NULL when capture is not possible, and then never tried again for this context).
+// A graph of n steps from buffer `cur`, and of the check of a whole residual interval, in *slot
+// (captured on first use; NULL when capture is not possible, and then never tried again for
+// this context).
 #ifndef LBM_STEP_GRAPHS
 #define LBM_STEP_GRAPHS 1
 #endif
 template <typename S>
-static cudaGraphExec_t step_graph(lbm_ctx* c, const ParamsOf<S>& p, int cur) {
+static cudaGraphExec_t step_graph(lbm_ctx* c, const ParamsOf<S>& p, int cur, int64_t n, bool check,
+                                  cudaGraphExec_t* slot) {
     if (!LBM_STEP_GRAPHS || c->graphs_failed) return nullptr;
-    if (c->step_graph[cur]) return c->step_graph[cur];
-    const int R = c->opt.residual_interval;
+    if (*slot) return *slot;
     bool ok = c->capture || cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) == cudaSuccess;
     cudaGraph_t g = nullptr;
     if (ok) ok = cudaStreamBeginCapture(c->capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
         int b = cur;
         cudaError_t e = cudaSuccess;
-        for (int i = 1; i <= R && e == cudaSuccess; ++i, b ^= 1) e = enqueue_step<S>(c, p, b, i, c->capture);
+        for (int64_t i = 0; i < n && e == cudaSuccess; ++i, b ^= 1) e = launch_step<S>(c->dev, b, p, c->capture);
+        if (e == cudaSuccess && check) e = enqueue_check<S>(c, p, b, 0, c->capture);
         const cudaError_t e2 = cudaStreamEndCapture(c->capture, &g);
         ok = e == cudaSuccess && e2 == cudaSuccess && g;
     }
-    if (ok) ok = cudaGraphInstantiate(&c->step_graph[cur], g, 0) == cudaSuccess;
+    if (ok) ok = cudaGraphInstantiate(slot, g, 0) == cudaSuccess;
     if (g) cudaGraphDestroy(g);
     if (!ok) {
-        c->step_graph[cur] = nullptr;
+        *slot = nullptr;
         c->graphs_failed = true;
         cudaGetLastError();  // a failed capture leaves no error behind for the next launch
     }
-    return c->step_graph[cur];
+    return *slot;
+}
+
+// Steps up to the next check launched one by one, or as one graph when the run before them was as
+// long: a program that advances a small cavity a few steps at a time spends most of such a call
+// in the launches (10 steps and the fields at 24^3: 81 -> 77 us a call).
+constexpr int64_t kRunMin = 4, kRunMax = 128;
+template <typename S>
+static int run_part(lbm_ctx* c, const ParamsOf<S>& p, int64_t n) {
+    const bool again = n >= kRunMin && n <= kRunMax && n == c->last_run;
+    c->last_run = n;
+    cudaGraphExec_t g = nullptr;
+    if (again) {
+        if (c->run_len != n) {
+            if (c->run_graph[0] || c->run_graph[1]) {  // the last run of the old length may still be at work
+                const int rc = wait_stream(c);
+                if (rc != LBM_OK) return rc;
+            }
+            for (cudaGraphExec_t& old : c->run_graph) {
+                if (old) cudaGraphExecDestroy(old);
+                old = nullptr;
+            }
+            c->run_len = n;
+        }
+        g = step_graph<S>(c, p, c->cur, n, false, &c->run_graph[c->cur]);
+    }
+    if (g) {
+        CUDA_OR_FAIL(c, cudaGraphLaunch(g, c->stream));
+        c->cur ^= (int)(n & 1);
+        c->steps += n;
+        return LBM_OK;
+    }
+    for (int64_t s = 0; s < n; ++s) {
+        CUDA_OR_FAIL(c, launch_step<S>(c->dev, c->cur, p, c->stream));
+        c->cur ^= 1;
+        c->steps += 1;
+    }
+    return LBM_OK;
 }
 
 template <typename S>
@@ -406,7 +443,7 @@ static int run_steps(lbm_ctx* c, int64_t n, bool* checked) {
     for (int64_t s = 0; s < n;) {
         // whole residual intervals, aligned with the step count, go as one graph launch
         if (R > 0 && c->steps % R == 0 && n - s >= R) {
-            if (cudaGraphExec_t g = step_graph<S>(c, p, c->cur)) {
+            if (cudaGraphExec_t g = step_graph<S>(c, p, c->cur, R, true, &c->step_graph[c->cur])) {
                 CUDA_OR_FAIL(c, cudaGraphLaunch(g, c->stream));
                 if (R & 1) c->cur ^= 1;
                 c->steps += R;
@@ -415,10 +452,11 @@ static int run_steps(lbm_ctx* c, int64_t n, bool* checked) {
                 continue;
             }
         }
-        CUDA_OR_FAIL(c, enqueue_step<S>(c, p, c->cur, c->steps + 1, c->stream));
-        c->cur ^= 1;
-        c->steps += 1;
-        s += 1;
+        const int64_t m = R > 0 ? std::min<int64_t>(n - s, R - c->steps % R) : n - s;
+        const int rc = run_part<S>(c, p, m);
+        if (rc != LBM_OK) return rc;
+        s += m;
+        CUDA_OR_FAIL(c, enqueue_check<S>(c, p, c->cur, c->steps, c->stream));
         if (R > 0 && c->steps % R == 0) *checked = true;
     }
     return LBM_OK;
@@ -862,8 +900,8 @@ void lbm::destroy_context(lbm_ctx* c) {
     {
         DeviceGuard g(c->device);
         wait_stream(c);
-        for (cudaGraphExec_t& g : c->step_graph)
-            if (g) cudaGraphExecDestroy(g);
+        for (cudaGraphExec_t* g : {&c->step_graph[0], &c->step_graph[1], &c->run_graph[0], &c->run_graph[1]})
+            if (*g) cudaGraphExecDestroy(*g);
         if (c->capture) cudaStreamDestroy(c->capture);
         if (c->imposed) cudaFree(c->imposed);
         if (c->own_arena && c->arena) cudaFree(c->arena);

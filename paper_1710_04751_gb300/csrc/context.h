@@ -55,6 +55,9 @@ struct lbm_ctx {
     // one per starting buffer, captured on a private stream when first needed
     cudaStream_t capture = nullptr;
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
+    // ... and, once a shorter run of steps is asked for twice in a row, run_len steps likewise
+    cudaGraphExec_t run_graph[2] = {nullptr, nullptr};
+    int64_t run_len = 0, last_run = 0;
     bool graphs_failed = false;  // capture not possible here: launch the steps one by one
     // state_fits_l2 of everything a step goes through: this context, the batch or all slabs
     bool in_l2 = false;

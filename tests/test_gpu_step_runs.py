@@ -1,0 +1,25 @@
+"""lbm_step in short runs of equal and changing lengths (the run graphs) against one long call:
+the same states, step counts and residuals, in every storage form, odd and even run lengths,
+with and without residual checks."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2, 3])
+@pytest.mark.parametrize("interval", [0, 7, 20])
+def test_runs_of_steps_equal_one_call(precision, interval):
+    import paper_1710_04751_gb300 as lbm
+    kw = dict(Ra=2e3, precision=precision, noise_amp=0.1, residual_interval=interval)
+    runs = [5] * 4 + [6] * 3 + [5, 5, 130, 130, 4, 4, 4, 3, 3, 1, 1, 20, 20, 20]
+    a, b = lbm.LBM((12, 9, 7), 15, **kw), lbm.LBM((12, 9, 7), 15, **kw)
+    for n in runs:
+        a.step(n)
+    b.step(sum(runs))
+    assert a.steps_done == b.steps_done == sum(runs)
+    assert a.residual() == b.residual()
+    for x, y in zip(a.get_populations(), b.get_populations()):
+        assert np.array_equal(x, y)
+    a.close()
+    b.close()
