@@ -90,10 +90,12 @@ __device__ __forceinline__ void batch_node(const BatchMember<S>& m, const Params
     const S* Gin = m.G[parity];
     S* Fout = m.F[parity ^ 1];
     S* Gout = m.G[parity ^ 1];
-    if (m.fast && j >= 1 && j + 1 < ny && k >= 1 && k + 1 < p.nz)
-        cavity_node<S, Q, true, UNIT>(Fin, Gin, nullptr, Fout, Gout, nullptr, p, i, j, k);
+    if (!m.fast)
+        cavity_node<S, Q, kAnyNode, UNIT>(Fin, Gin, nullptr, Fout, Gout, nullptr, p, i, j, k);
+    else if (j >= 1 && j + 1 < ny && k >= 1 && k + 1 < p.nz)
+        cavity_node<S, Q, kInterior, UNIT>(Fin, Gin, nullptr, Fout, Gout, nullptr, p, i, j, k);
     else
-        cavity_node<S, Q, false, UNIT>(Fin, Gin, nullptr, Fout, Gout, nullptr, p, i, j, k);
+        cavity_node<S, Q, kWall, UNIT>(Fin, Gin, nullptr, Fout, Gout, nullptr, p, i, j, k);
 }
 
 // Parameters of a member of a sweep: every field of `base` (a kernel parameter, so it

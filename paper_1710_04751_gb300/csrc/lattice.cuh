@@ -30,6 +30,15 @@ __host__ __device__ inline int dir_index(int dx, int dy, int dz) {
     return dz > 0 ? 5 : 6;
 }
 
+// direction a with e_y (flip & 1) and e_z (flip & 2) reversed
+__host__ __device__ constexpr int mirror(int a, int flip) {
+    const int dy = flip & 1 ? -ey(a) : ey(a), dz = flip & 2 ? -ez(a) : ez(a);
+    return a >= 7 ? 7 + (ex(a) < 0) + 2 * (dy < 0) + 4 * (dz < 0)
+         : ex(a) != 0 ? a
+         : ey(a) != 0 ? (dy > 0 ? 3 : 4)
+         : ez(a) != 0 ? (dz > 0 ? 5 : 6) : 0;
+}
+
 // D3Q15 collision matrix entry K_b(e_a) (Sec. 2.2, the Gram-Schmidt basis K_0..K_14).
 __host__ __device__ constexpr int k15(int b, int a) {
     return b == 0 ? 1

@@ -120,6 +120,46 @@ __device__ __forceinline__ void pull(const S* __restrict__ Fin, const S* __restr
     }
 }
 
+// Pull of a cavity node (boundary 0) at a y or z wall: the rules of pull with every link's source
+// chosen by selects, so that all loads of the node are in flight together.  (pull branches per
+// link; the rows at the walls, a sixth of a 24^3 cavity's, then waited for memory link by link and
+// set the length of the whole step.)  Per step before / now: FP32 D3Q15 16^3 5.3 / 2.1 us, 32^3
+// 6.3 / 2.4, 64^3 11.1 / 8.5, 128^3 78.0 / 75.7; FP16 64^3 17.4 / 8.8, 128^3 68.8 / 54.4; BF16
+// 128^3 70.6 / 54.7; FP64 16^3 16.0 / 12.8, 32^3 24.6 / 23.4.
+template <typename S, int Q>
+__device__ __forceinline__ void pull_wall(const S* __restrict__ Fin, const S* __restrict__ Gin,
+                                          const float* __restrict__ Tin, const ParamsOf<S>& p, int i, int j,
+                                          int k, int c, typename Storage<S>::real (&f)[15],
+                                          typename Storage<S>::real (&g)[Q]) {
+    using real = typename Storage<S>::real;
+    using St = Storage<S>;
+    const int nx = p.nx, nxy = nx * p.ny, P = (int)p.plane;
+    const bool xl = i == 0, xh = i == nx - 1, yl = j == 0, yh = j == p.ny - 1, zl = k == 0, zh = k == p.nz - 1;
+    const bool specular = p.adiabatic_mode == 1;
+#pragma unroll
+    for (int a = 0; a < 15; ++a) {
+        const bool xo = ex(a) > 0 ? xl : ex(a) < 0 && xh;  // the link comes through a wall of this axis
+        const bool yo = ey(a) > 0 ? yl : ey(a) < 0 && yh;
+        const bool zo = ez(a) > 0 ? zl : ez(a) < 0 && zh;
+        const int dx = ex(a), dy = ey(a) * nx, dz = ez(a) * nxy;
+        const bool out = xo || yo || zo;
+        f[a] = St::load_f(Fin[out ? opp(a) * P + c : a * P + (c - dx - dy - dz)], p.wf[a]);
+        if (a < Q) {
+            // population and node the scalar link takes: its own; mirrored at the y and z walls it
+            // crosses; reversed at this node (x faces, and every wall in the bounce-back form)
+            int b = a, node = c - dx - dy - dz;
+            if (ey(a) != 0 && yo) b = mirror(a, 1), node += dy;
+            if (ez(a) != 0 && zo) b = ey(a) != 0 && yo ? mirror(a, 3) : mirror(a, 2), node += dz;
+            const bool back = xo || (!specular && (yo || zo));
+            b = back ? opp(a) : b;
+            node = back ? c : node;
+            const real v = St::load(Gin[b * P + node], thermal_offset<S>(Tin, p, a, node));
+            const real Tw = ex(a) > 0 ? p.T_cold : p.T_hot;
+            g[a] = xo ? -v + real(2) * p.wg[a] * Tw : v;
+        }
+    }
+}
+
 // Macroscopic variables, both collisions and the store of one node.  UNIT: the paper's
 // unit higher-order rates (collide_unit.cuh), for which the post-collision state needs
 // only the low-order moments of the pulled populations.
@@ -246,7 +286,8 @@ __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15]
 // ---------------------------------------------------------------------------------
 // ONCE: load_pop's first form (the batched kernels, whose members together seldom fit into L2
 // and whose register budget is tight, load plainly).
-template <typename S, int Q, bool INTERIOR, bool UNIT = false, bool IMPOSE = false, bool ONCE = false>
+enum Place { kAnyNode, kInterior, kWall };  // kInterior, kWall: boundary 0 and 32-bit node indices
+template <typename S, int Q, Place PLACE, bool UNIT = false, bool IMPOSE = false, bool ONCE = false>
 __device__ __forceinline__ void cavity_node(const S* __restrict__ Fin, const S* __restrict__ Gin,
                                             const float* __restrict__ Tin, S* __restrict__ Fout,
                                             S* __restrict__ Gout, float* __restrict__ Tout,
@@ -260,7 +301,7 @@ __device__ __forceinline__ void cavity_node(const S* __restrict__ Fin, const S* 
     const int64_t c = k * nxy + (int64_t)j * nx + i;
     const int64_t P = p.plane;
     real f[15], g[Q];
-    if constexpr (INTERIOR) {
+    if constexpr (PLACE == kInterior) {
         uint64_t once = 0;
         if constexpr (ONCE && sizeof(S) == 4) once = once_policy(p.in_l2);
         const bool lo = i == 0, hi = i == nx - 1;
@@ -291,6 +332,8 @@ __device__ __forceinline__ void cavity_node(const S* __restrict__ Fin, const S* 
             const S* Fa = Fin + (int64_t)a * P - shift;
             f[a] = St::load_f(load_pop<S, ONCE>(Fa + (out ? ci + shift + (opp(a) - a) * Pi : ci), once), p.wf[a]);
         }
+    } else if constexpr (PLACE == kWall) {
+        pull_wall<S, Q>(Fin, Gin, Tin, p, i, j, k, (int)c, f, g);
     } else {
         pull<S, Q>(Fin, Gin, Tin, p, i, j, k, c, f, g);
     }

@@ -74,9 +74,9 @@ __global__ void __launch_bounds__(128, (cavity_min_blocks<S, Q>() - (IMPOSE && c
     if (i >= p.nx) return;
     const bool interior = j >= 1 && j + 1 < p.ny && k >= 1 && k + 1 < p.nz;
     if (interior)
-        cavity_node<S, Q, true, UNIT, IMPOSE, true>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
+        cavity_node<S, Q, kInterior, UNIT, IMPOSE, true>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
     else
-        cavity_node<S, Q, false, UNIT, IMPOSE, true>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
+        cavity_node<S, Q, kWall, UNIT, IMPOSE, true>(Fin, Gin, Tin, Fout, Gout, Tout, p, i, j, k, step, imposed);
 }
 
 // ---------------------------------------------------------------------------------
@@ -161,7 +161,7 @@ __device__ __forceinline__ void pair_row(const S* __restrict__ Fin, const S* __r
     } else {
 #pragma unroll 1
         for (int e = 0; e < 2; ++e)
-            cavity_node<S, Q, false, UNIT>(Fin, Gin, Tin, Fout, Gout, Tout, p, 2 * t + e, j, k, step);
+            cavity_node<S, Q, kWall, UNIT>(Fin, Gin, Tin, Fout, Gout, Tout, p, 2 * t + e, j, k, step);
     }
 }
 
