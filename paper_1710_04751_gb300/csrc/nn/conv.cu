@@ -684,10 +684,12 @@ __global__ void __launch_bounds__(128, 1)
 // ---------------------------------------------------------------------------------
 constexpr int W9_N = 96;                    // columns of one ky: 3 kx of 32 output channels
 constexpr int W9_ROWS = 64 * 64;            // bytes of 64 voxels of 32 channels
-constexpr int W9_SLOT = 7 * W9_ROWS;        // four chunks of X, three copies of dZ
+constexpr int W9_X = 4 * W9_ROWS;           // a ring slot's four chunks of X
+constexpr int W9_Z = 3 * W9_ROWS;           // and its three copies of dZ
 constexpr int W9_SLOTS = 7;
+constexpr int W9_RING = W9_SLOTS * (W9_X + W9_Z);  // the X slots, then the dZ slots
 constexpr int W9_SUM = 128 * 3 * W9_N * 4;  // bytes of one CTA's accumulators
-static_assert(W9_SLOTS * W9_SLOT >= W9_SUM, "the pair's sums go where the ring was");
+static_assert(W9_RING >= W9_SUM, "the pair's sums go where the ring was");
 
 struct Wgrad9Args {
     int N, cin, n;       // output channels, input channels, grid edge
@@ -738,7 +740,7 @@ __global__ void __launch_bounds__(128, 1)
     extern __shared__ uint8_t w9_smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(w9_smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * W9_SLOT);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + W9_RING);
     uint64_t* empty = full + S;
     uint64_t* done = empty + S;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
@@ -787,7 +789,8 @@ __global__ void __launch_bounds__(128, 1)
                 failed = 1;
                 break;
             }
-            uint8_t* a = smem + s * W9_SLOT;
+            uint8_t* a = smem + s * W9_X;
+            uint8_t* z = smem + S * W9_X + s * W9_Z;
             const int x0 = w.seg * 64, y0 = w.y * RB, yz = y0 + 1 - w.left * RB;  // dZ rows yz .. yz + RB - 1
             if (elected) {
                 mbar_expect_tx(full + s, (w.data() ? 7 : 3) * W9_ROWS);
@@ -798,17 +801,18 @@ __global__ void __launch_bounds__(128, 1)
                 }
 #pragma unroll
                 for (int kx = 0; kx < 3; ++kx)
-                    tma_load_5d(a + (4 + kx) * W9_ROWS, &tmZ, full + s, n0, x0 + 1 - kx, yz, w.z, w.b);
+                    tma_load_5d(z + kx * W9_ROWS, &tmZ, full + s, n0, x0 + 1 - kx, yz, w.z, w.b);
             }
             ++issued;
             if (++s == S) s = 0, ph ^= 1u;
         }
     } else if (nst > 0 && warp == 1) {
         const bool elected = elect_lane();
-        const uint32_t idesc = idesc_bf16_f32_mn(CBM, W9_N);
+        const uint32_t idesc = idesc_bf16_f32_mn(CBM, W9_N), idesc2 = idesc_bf16_f32_mn(CBM, 2 * W9_N);
         const uint32_t ahi = (uint32_t)(sdesc_mn(0, W9_ROWS, 512, 4) >> 32);
-        const uint32_t ring = (uint32_t)sdesc_mn(smem_u32(smem), W9_ROWS, 512, 4);
-        uint32_t acc = 0, z[3] = {ring, ring, ring};  // dZ of this slot, of the one before, of two before
+        const uint32_t xring = (uint32_t)sdesc_mn(smem_u32(smem), W9_ROWS, 512, 4);
+        const uint32_t zring = xring + (uint32_t)(S * W9_X >> 4);
+        uint32_t acc = 0;
         W9Walk w(first, nst, args.run, lead, args.segs, n);
         int s = 0, s1 = S - 1, s2 = S - 2;  // this slot and the ones before
         uint32_t ph = 0;
@@ -817,21 +821,34 @@ __global__ void __launch_bounds__(128, 1)
                 failed = 1;
                 break;
             }
-            const uint32_t a = ring + (uint32_t)(s * (W9_SLOT >> 4));
-            z[2] = z[1], z[1] = z[0], z[0] = a + (4 * W9_ROWS >> 4);
+            const uint32_t a = xring + (uint32_t)(s * (W9_X >> 4));
+            // the dZ of this slot, of the one before and of two before
+            const uint32_t z[3] = {zring + (uint32_t)(s * (W9_Z >> 4)), zring + (uint32_t)(s1 * (W9_Z >> 4)),
+                                   zring + (uint32_t)(s2 * (W9_Z >> 4))};
             tc_fence_after();
             if (elected && w.data()) {
+                // columns (2 - ky) 96 of the accumulators: tap ky
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {  // K = 16 per MMA: two atoms of 8 voxels
-                    constexpr int line = 64 / RB * 64;  // bytes of an x-row of the block
-                    const int row = kk * RB / 4;        // x-row of the block
+                    if constexpr (RB == 1) {
+                        // The taps' dZ rows are in three slots one after another in the ring: two that
+                        // don't straddle its end are one operand of six 32-channel groups.
+                        const bool old = s1 != 0;  // the older two, else the newer two
+                        mma_bf16(tmem + (old ? 0u : (uint32_t)W9_N), a + kk * 64, ahi, z[old ? 2 : 1] + kk * 64, ahi,
+                                 idesc2, acc);
+                        mma_bf16(tmem + (old ? 2u * W9_N : 0u), a + kk * 64, ahi, z[old ? 0 : 2] + kk * 64, ahi,
+                                 idesc, acc);
+                    } else {
+                        constexpr int line = 64 / RB * 64;  // bytes of an x-row of the block
+                        const int row = kk * RB / 4;        // x-row of the block
 #pragma unroll
-                    for (int ky = 0; ky < 3; ++ky) {
-                        // dZ row y0 + row - (ky - 1): place d = row - ky of this slot, or of one before
-                        const int back = row >= ky ? 0 : (ky - row + RB - 1) / RB;
-                        const int d = row - ky + back * RB;
-                        mma_bf16(tmem + (uint32_t)(ky * W9_N), a + kk * 64, ahi,
-                                        z[back] + (uint32_t)(((d - row) * line + kk * 1024) >> 4), ahi, idesc, acc);
+                        for (int ky = 0; ky < 3; ++ky) {
+                            // dZ row y0 + row - (ky - 1): place d = row - ky of this slot, or of one before
+                            const int back = row >= ky ? 0 : (ky - row + RB - 1) / RB;
+                            const int d = row - ky + back * RB;
+                            mma_bf16(tmem + (uint32_t)((2 - ky) * W9_N), a + kk * 64, ahi,
+                                     z[back] + (uint32_t)(((d - row) * line + kk * 1024) >> 4), ahi, idesc, acc);
+                        }
                     }
                     acc = 1;
                 }
@@ -892,7 +909,7 @@ __global__ void __launch_bounds__(128, 1)
                     v[4 * j + 3] += w.w;
                 }
             }
-            const int t = c >> 5, col0 = n0 + (c & 31);  // tap within kz (ky 3 + kx)
+            const int g = c >> 5, t = (2 - g / 3) * 3 + g % 3, col0 = n0 + (c & 31);  // t: tap (ky, kx) within kz
             float* C = slab + (int64_t)((kz * 9 + t) * args.cin + ci) * args.N + col0;
 #pragma unroll
             for (int j = 0; j < 4; ++j)  // N is a multiple of 8: whole quadruples
@@ -1048,7 +1065,7 @@ cudaError_t launch_wgrad9(const __nv_bfloat16* X, int B, int n, int cin, const _
         }
     const int per = (total + best_s * best_c - 1) / (best_s * best_c);
     *slices = (total + per * best_c - 1) / (per * best_c);  // every slice has work in its first CTA
-    constexpr int smem = 1024 + W9_SLOTS * W9_SLOT + 256;
+    constexpr int smem = 1024 + W9_RING + 256;
     const auto kernel = n == 16 ? conv_wgrad9_kernel<4> : n == 32 ? conv_wgrad9_kernel<2> : conv_wgrad9_kernel<1>;
     static std::once_flag once;
     static cudaError_t attr = cudaSuccess;
