@@ -197,6 +197,13 @@ __global__ void __launch_bounds__(128, 1)
     if (warp == 0) tmem_dealloc(tmem, L::TMEM_COLS);
 }
 
+// 32 bytes to a 32-byte boundary.
+__device__ __forceinline__ void store32(void* p, const uint32_t (&h)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(h[0]), "r"(h[1]), "r"(h[2]),
+                 "r"(h[3]), "r"(h[4]), "r"(h[5]), "r"(h[6]), "r"(h[7])
+                 : "memory");
+}
+
 // ---------------------------------------------------------------------------------
 // The same convolution with the three kx taps side by side in the MMA's N (16 <= n <= 128; the
 // kernel above takes the grids below and beyond).
@@ -223,9 +230,57 @@ struct X3Args {
     int mode;
     void* C;
     const float* bias;
+    int wide;  // rows of C start on 32 bytes and hold whole 16-column chunks
     int* err;
 };
 constexpr int kX3Threads = 320;  // producer, MMA, two sets of four epilogue warps
+
+constexpr int kX3Bias = 304;     // output channels in whole tiles, at most: 6 tiles of 48 and a chunk
+
+// The store of 16 output channels of a row, bias and ReLU applied.  In 32-byte pieces where the
+// rows allow it: a lane's row is a sector of its own, which two 16-byte stores write twice.
+__device__ __forceinline__ void x3_store16(const X3Args& a, int row, int col0, const float (&v)[16]) {
+    if (col0 >= a.N) return;
+    if (a.mode == CONV_BIAS_RELU_BF16) {
+        __nv_bfloat16* C = static_cast<__nv_bfloat16*>(a.C) + (int64_t)row * a.N + col0;
+        uint32_t h[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+            h[j] = *reinterpret_cast<const uint32_t*>(&b);
+        }
+        if (a.wide) {
+            store32(C, h);
+        } else if (a.N % 8 == 0) {
+            reinterpret_cast<uint4*>(C)[0] = make_uint4(h[0], h[1], h[2], h[3]);
+            if (col0 + 8 < a.N) reinterpret_cast<uint4*>(C)[1] = make_uint4(h[4], h[5], h[6], h[7]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (col0 + j < a.N) C[j] = __float2bfloat16_rn(v[j]);
+        }
+    } else {
+        float* C = static_cast<float*>(a.C) + (int64_t)row * a.N + col0;
+        if (a.wide) {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uint32_t h[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) h[j] = __float_as_uint(v[8 * q + j]);
+                store32(C + 8 * q, h);
+            }
+        } else if (a.N % 8 == 0) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (col0 + 4 * j < a.N)
+                    reinterpret_cast<float4*>(C)[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+                if (col0 + j < a.N) C[j] = v[j];
+        }
+    }
+}
 
 // One item's place: first row, grid position, output channels, the kz planes inside the grid.
 struct X3Item {
@@ -244,9 +299,14 @@ struct X3Item {
 // the other.  (With a CTA per item, two on an SM, the 64^3 96 -> 32 layer, batch 2, spent 25 of
 // 87 us in 2048 CTAs' set-up and 22 in epilogues.)  Per call with the host wait, that form / this
 // one: that layer 110 / 92 us, 64^3 32 -> 32 77 / 64, 32^3 64 -> 192 in FP32 80 / 68, 128^3
-// 32 -> 32 234 / 169, 16^3 128 -> 128 (an item per CTA) 35 / 35.  The tensor pipe is then 70% busy
-// with operand reads (67 cycles per MMA of 96 columns); sharing the weights in clusters of two
-// by TMA multicast was no faster.
+// 32 -> 32 234 / 169, 16^3 128 -> 128 (an item per CTA) 35 / 35.  A 96 -> 32 item takes 66 cycles per
+// MMA of 96 columns (48 of math); leaving out either the weights' or the input's loads changes
+// that little, and neither sharing the weights in clusters of two by TMA multicast nor pairs of
+// CTAs with MMAs of M = 256 (-2 to -10% from 64 input channels on, +20% at 32) was worth a second
+// form.  With 32 input channels the epilogue is the longer part: the rows' ends go between warps
+// as quadruples that every lane reads, the bias comes from shared memory, and a lane's channels
+// are stored as whole 32-byte sectors.  Before / after those: 64^3 batch 2 32 -> 32 63 / 59 us and
+// in FP32 73 / 68, 128^3 FP32 233 / 203, 32^3 64 -> 192 FP32 67 / 62.
 template <int BN>
 __global__ void __launch_bounds__(kX3Threads, 1)
     conv_x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmW,
@@ -262,12 +322,17 @@ __global__ void __launch_bounds__(kX3Threads, 1)
     uint64_t* done = acc_empty + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     __shared__ volatile int failed;
-    __shared__ float edge[2][2][4][2][16];  // of each epilogue set: P_0 of a warp's last row, P_2 of its first
+    __shared__ float4 edge[2][2][4][2][4];  // of each epilogue set: P_0 of a warp's last row, P_2 of its first
     constexpr int W = 3 * BN, B_TILE = BN * 64;
+
+    __shared__ float4 bias[kX3Bias / 4];
 
     if (*static_cast<volatile int*>(args.err) != 0) return;  // another CTA timed out
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const int MT = args.mt, n = args.n;
+    if (args.mode == CONV_BIAS_RELU_BF16)
+        for (int c = threadIdx.x; c < kX3Bias; c += kX3Threads)
+            reinterpret_cast<float*>(bias)[c] = c < args.N ? args.bias[c] : 0.f;
 
     if (threadIdx.x == 0) {
         failed = 0;
@@ -387,33 +452,53 @@ __global__ void __launch_bounds__(kX3Threads, 1)
                 tmem_landed(p0);
                 tmem_landed(v);
                 tmem_landed(p2);
-                if (n > 32) {  // block-uniform
-                    float(&e)[4][2][16] = edge[set][par];
+                float l[16], r[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    l[j] = __shfl_up_sync(0xffffffffu, p0[j], 1);
+                    r[j] = __shfl_down_sync(0xffffffffu, p2[j], 1);
+                }
+                if (n > 32) {  // block-uniform: an x-row spans warps
+                    float4(&e)[4][2][4] = edge[set][par];
                     if (lane == 31) {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) e[quarter][0][j] = p0[j];
+                        for (int j = 0; j < 4; ++j)
+                            e[quarter][0][j] = make_float4(p0[4 * j], p0[4 * j + 1], p0[4 * j + 2], p0[4 * j + 3]);
                     }
                     if (lane == 0) {
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) e[quarter][1][j] = p2[j];
+                        for (int j = 0; j < 4; ++j)
+                            e[quarter][1][j] = make_float4(p2[4 * j], p2[4 * j + 1], p2[4 * j + 2], p2[4 * j + 3]);
                     }
                     bar_sync(1 + set, 128);
+                    // every lane reads (one address per warp) and the lanes at the warp's ends take it
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        float l = __shfl_up_sync(0xffffffffu, p0[j], 1), r = __shfl_down_sync(0xffffffffu, p2[j], 1);
-                        if (lane == 0 && !first) l = e[quarter - 1][0][j];
-                        if (lane == 31 && !last) r = e[quarter + 1][1][j];
-                        v[j] += (first ? 0.f : l) + (last ? 0.f : r);
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float l = __shfl_up_sync(0xffffffffu, p0[j], 1);
-                        const float r = __shfl_down_sync(0xffffffffu, p2[j], 1);
-                        v[j] += (first ? 0.f : l) + (last ? 0.f : r);
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 el = e[(quarter + 3) & 3][0][j], er = e[(quarter + 1) & 3][1][j];
+                        l[4 * j] = lane == 0 ? el.x : l[4 * j];
+                        l[4 * j + 1] = lane == 0 ? el.y : l[4 * j + 1];
+                        l[4 * j + 2] = lane == 0 ? el.z : l[4 * j + 2];
+                        l[4 * j + 3] = lane == 0 ? el.w : l[4 * j + 3];
+                        r[4 * j] = lane == 31 ? er.x : r[4 * j];
+                        r[4 * j + 1] = lane == 31 ? er.y : r[4 * j + 1];
+                        r[4 * j + 2] = lane == 31 ? er.z : r[4 * j + 2];
+                        r[4 * j + 3] = lane == 31 ? er.w : r[4 * j + 3];
                     }
                 }
-                conv_store16(args.C, args.N, args.mode, args.bias, it.m0 + t * CBM + quarter * 32 + lane, it.n0 + c, v);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] += (first ? 0.f : l[j]) + (last ? 0.f : r[j]);
+                const int row = it.m0 + t * CBM + quarter * 32 + lane, col0 = it.n0 + c;
+                if (args.mode == CONV_BIAS_RELU_BF16) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 bj = bias[(col0 >> 2) + j];
+                        v[4 * j] = fmaxf(v[4 * j] + bj.x, 0.f);
+                        v[4 * j + 1] = fmaxf(v[4 * j + 1] + bj.y, 0.f);
+                        v[4 * j + 2] = fmaxf(v[4 * j + 2] + bj.z, 0.f);
+                        v[4 * j + 3] = fmaxf(v[4 * j + 3] + bj.w, 0.f);
+                    }
+                }
+                x3_store16(args, row, col0, v);
             }
             tc_fence_before();
             if (lane == 0) mbar_arrive(acc_empty + (k & 1));
@@ -677,6 +762,13 @@ __global__ void __launch_bounds__(128, 1)
 // rows y0 - 1 .. y0 + RB from this slot and the one or two before it, so that each dZ row is
 // loaded once per kx.  A run of blocks that starts (at a plane's or the range's first block)
 // is led in by slots with dZ rows only.
+// Operand reads and fills of shared memory bound the kernel, not the tensor pipe: per 16 voxels
+// three MMAs read 3 (4 + 3) KB and the fill adds 7, 219 cycles at 128 bytes a cycle against 144
+// of math.  The dZ slots lie one after another, so from n = 64 on the rows of two ky taps are one
+// operand of N = 192 and the A tile is read twice, not three times.  Calls with the host wait,
+// three MMAs / two: 64^3 batch 2, 96 -> 32 channels 187 / 163 us, batch 4 535 / 437, 128^3
+// 32 -> 32 370 / 304, 64^3 64 -> 64 118 / 105.  (Below 64 a slot holds several rows, which would
+// take a box per row and kx.)
 // The accumulators fill 288 tensor-memory columns: a CTA holds one M tile of 32 output
 // channels and a range of the blocks; where that leaves SMs idle, two CTAs of a cluster share a
 // range and the second adds its sums to the first's through distributed shared memory (a fixed
@@ -1027,7 +1119,7 @@ cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const _
             !make_w_map(&tw, W, cout, 27 * cin, ldw, 32, bn))
             return cudaErrorInvalidValue;
         X3Args a{cout, n, cin / 32, cin, ntiles, (int)(tiles / mt) * ntiles, by1, mt, (mt * by1 + 2) * n * 64, stage,
-                 std::min(8, kX3Smem / stage), mode, out, bias, err};
+                 std::min(8, kX3Smem / stage), mode, out, bias, cout % 16 == 0 && !((uintptr_t)out & 31), err};
         switch (bn) {
         case 16: return launch_x3<16>(tx, tw, a, st);
         case 32: return launch_x3<32>(tx, tw, a, st);
@@ -1113,7 +1205,7 @@ cudaError_t conv_wgrad_implicit(const __nv_bfloat16* X, int B, int n, int cin, c
     const int mtiles = (Kp + CBM - 1) / CBM;
     if ((size_t)used * Kp * cout > ws_floats) return cudaErrorInvalidValue;
     // The nine-tap form where it measured faster (calls with the host wait, us, one-tap / nine-tap):
-    // 64^3 batch 2, 96 -> 32 channels 286 / 190 and 32 -> 32 136 / 108, 32^3 batch 2, 192 -> 64
+    // 64^3 batch 2, 96 -> 32 channels 286 / 163 and 32 -> 32 136 / 101, 32^3 batch 2, 192 -> 64
     // 117 / 101; below that its long ramp shows: 32^3, 64 -> 64 79 / 82, 16^3 batch 4, 64 -> 48
     // 64 / 75.  More than 64 output channels fill the one-tap form's MMAs.
     if (n >= 16 && cout <= 64 && M * cin >= (int64_t(1) << 23)) {
