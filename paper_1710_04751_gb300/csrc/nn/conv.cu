@@ -764,11 +764,11 @@ __global__ void __launch_bounds__(128, 1)
 // is led in by slots with dZ rows only.
 // Operand reads and fills of shared memory bound the kernel, not the tensor pipe: per 16 voxels
 // three MMAs read 3 (4 + 3) KB and the fill adds 7, 219 cycles at 128 bytes a cycle against 144
-// of math.  The dZ slots lie one after another, so from n = 64 on the rows of two ky taps are one
-// operand of N = 192 and the A tile is read twice, not three times.  Calls with the host wait,
-// three MMAs / two: 64^3 batch 2, 96 -> 32 channels 187 / 163 us, batch 4 535 / 437, 128^3
-// 32 -> 32 370 / 304, 64^3 64 -> 64 118 / 105.  (Below 64 a slot holds several rows, which would
-// take a box per row and kx.)
+// of math.  The dZ rows lie one after another in their ring, [row][kx], so the rows of two ky taps
+// are one operand of N = 192 and the A tile is read twice, not three times.  Calls with the host
+// wait, three MMAs / two: 64^3 batch 2, 96 -> 32 channels 187 / 163 us, batch 4 535 / 437, 128^3
+// 32 -> 32 370 / 304, 64^3 64 -> 64 118 / 105, 32^3 batch 4, 96 -> 64 125 / 117,
+// batch 2, 192 -> 64 103 / 97.
 // The accumulators fill 288 tensor-memory columns: a CTA holds one M tile of 32 output
 // channels and a range of the blocks; where that leaves SMs idle, two CTAs of a cluster share a
 // range and the second adds its sums to the first's through distributed shared memory (a fixed
@@ -777,7 +777,7 @@ __global__ void __launch_bounds__(128, 1)
 constexpr int W9_N = 96;                    // columns of one ky: 3 kx of 32 output channels
 constexpr int W9_ROWS = 64 * 64;            // bytes of 64 voxels of 32 channels
 constexpr int W9_X = 4 * W9_ROWS;           // a ring slot's four chunks of X
-constexpr int W9_Z = 3 * W9_ROWS;           // and its three copies of dZ
+constexpr int W9_Z = 3 * W9_ROWS;           // and its dZ rows, three copies each
 constexpr int W9_SLOTS = 7;
 constexpr int W9_RING = W9_SLOTS * (W9_X + W9_Z);  // the X slots, then the dZ slots
 constexpr int W9_SUM = 128 * 3 * W9_N * 4;  // bytes of one CTA's accumulators
@@ -845,6 +845,7 @@ __global__ void __launch_bounds__(128, 1)
     const int first = blockIdx.x * args.per;  // the pair's CTAs take consecutive ranges
     const int nst = max(0, min(args.per, args.total - first));
     constexpr int lead = RB == 1 ? 2 : 1;
+    constexpr int line = W9_ROWS / RB;        // bytes of an x-row of the block
     const int gpt = args.cin >> 5;            // channel groups per kz
 
     if (threadIdx.x == 0) {
@@ -892,8 +893,8 @@ __global__ void __launch_bounds__(128, 1)
                         tma_load_5d(a + q * W9_ROWS, &tmX, full + s, gc[q], x0, y0, w.z + gz[q], w.b);
                 }
 #pragma unroll
-                for (int kx = 0; kx < 3; ++kx)
-                    tma_load_5d(z + kx * W9_ROWS, &tmZ, full + s, n0, x0 + 1 - kx, yz, w.z, w.b);
+                for (int q = 0; q < 3 * RB; ++q)
+                    tma_load_5d(z + q * line, &tmZ, full + s, n0, x0 + 1 - q % 3, yz + q / 3, w.z, w.b);
             }
             ++issued;
             if (++s == S) s = 0, ph ^= 1u;
@@ -903,7 +904,9 @@ __global__ void __launch_bounds__(128, 1)
         const uint32_t idesc = idesc_bf16_f32_mn(CBM, W9_N), idesc2 = idesc_bf16_f32_mn(CBM, 2 * W9_N);
         const uint32_t ahi = (uint32_t)(sdesc_mn(0, W9_ROWS, 512, 4) >> 32);
         const uint32_t xring = (uint32_t)sdesc_mn(smem_u32(smem), W9_ROWS, 512, 4);
-        const uint32_t zring = xring + (uint32_t)(S * W9_X >> 4);
+        // dZ: a ring of x-rows, [row][kx][voxel]
+        const uint32_t zring = (uint32_t)sdesc_mn(smem_u32(smem + S * W9_X), line, 512, 4);
+        constexpr int ROWS = S * RB;
         uint32_t acc = 0;
         W9Walk w(first, nst, args.run, lead, args.segs, n);
         int s = 0, s1 = S - 1, s2 = S - 2;  // this slot and the ones before
@@ -914,34 +917,24 @@ __global__ void __launch_bounds__(128, 1)
                 break;
             }
             const uint32_t a = xring + (uint32_t)(s * (W9_X >> 4));
-            // the dZ of this slot, of the one before and of two before
-            const uint32_t z[3] = {zring + (uint32_t)(s * (W9_Z >> 4)), zring + (uint32_t)(s1 * (W9_Z >> 4)),
-                                   zring + (uint32_t)(s2 * (W9_Z >> 4))};
+            // RB = 1: the dZ of this slot, of the one before and of two before
+            const uint32_t zs[3] = {zring + (uint32_t)(s * (W9_Z >> 4)), zring + (uint32_t)(s1 * (W9_Z >> 4)),
+                                    zring + (uint32_t)(s2 * (W9_Z >> 4))};
             tc_fence_after();
             if (elected && w.data()) {
-                // columns (2 - ky) 96 of the accumulators: tap ky
+                // tap ky takes the dZ row ky rows before this one into the columns (2 - ky) 96; two rows
+                // that don't straddle the ring's end are one operand of six 32-channel groups
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {  // K = 16 per MMA: two atoms of 8 voxels
-                    if constexpr (RB == 1) {
-                        // The taps' dZ rows are in three slots one after another in the ring: two that
-                        // don't straddle its end are one operand of six 32-channel groups.
-                        const bool old = s1 != 0;  // the older two, else the newer two
-                        mma_bf16(tmem + (old ? 0u : (uint32_t)W9_N), a + kk * 64, ahi, z[old ? 2 : 1] + kk * 64, ahi,
-                                 idesc2, acc);
-                        mma_bf16(tmem + (old ? 2u * W9_N : 0u), a + kk * 64, ahi, z[old ? 0 : 2] + kk * 64, ahi,
-                                 idesc, acc);
-                    } else {
-                        constexpr int line = 64 / RB * 64;  // bytes of an x-row of the block
-                        const int row = kk * RB / 4;        // x-row of the block
-#pragma unroll
-                        for (int ky = 0; ky < 3; ++ky) {
-                            // dZ row y0 + row - (ky - 1): place d = row - ky of this slot, or of one before
-                            const int back = row >= ky ? 0 : (ky - row + RB - 1) / RB;
-                            const int d = row - ky + back * RB;
-                            mma_bf16(tmem + (uint32_t)((2 - ky) * W9_N), a + kk * 64, ahi,
-                                     z[back] + (uint32_t)(((d - row) * line + kk * 1024) >> 4), ahi, idesc, acc);
-                        }
-                    }
+                    const int row = s * RB + kk * RB / 4;
+                    const auto z = [&](int ky) {
+                        if constexpr (RB == 1) return zs[ky] + kk * 64;
+                        const int at = row >= ky ? row - ky : row - ky + ROWS;
+                        return zring + (uint32_t)((at * 3 * line + kk % (4 / RB) * 1024) >> 4);
+                    };
+                    const bool old = RB == 1 ? s1 != 0 : row != 1;  // the older two together, else the newer two
+                    mma_bf16(tmem + (old ? 0u : (uint32_t)W9_N), a + kk * 64, ahi, z(old ? 2 : 1), ahi, idesc2, acc);
+                    mma_bf16(tmem + (old ? 2u * W9_N : 0u), a + kk * 64, ahi, z(old ? 0 : 2), ahi, idesc, acc);
                     acc = 1;
                 }
             }
@@ -1168,7 +1161,7 @@ cudaError_t launch_wgrad9(const __nv_bfloat16* X, int B, int n, int cin, const _
     if (attr != cudaSuccess) return attr;
     const int bx = n < 64 ? n : 64, RB = 64 / bx, segs = n / bx;
     CUtensorMap tx, tz;
-    if (!make_x_map(&tx, X, B, n, cin, 32, bx, RB, 1, 1) || !make_x_map(&tz, dZ, B, n, cout, 32, bx, RB, 1, 1))
+    if (!make_x_map(&tx, X, B, n, cin, 32, bx, RB, 1, 1) || !make_x_map(&tz, dZ, B, n, cout, 32, bx, 1, 1, 1))
         return cudaErrorInvalidValue;
     const Wgrad9Args a{cout, cin, n, segs, n / RB, total, per, Kp, best_c == 2, ws, err};
     cudaLaunchConfig_t cfg = {};
