@@ -399,13 +399,21 @@ static cudaGraphExec_t step_graph(lbm_ctx* c, const ParamsOf<S>& p, int cur, int
     return *slot;
 }
 
+// Whether the caller is capturing the stream: it then takes launches, but no graph of ours.
+static bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // Steps up to the next check launched one by one, or as one graph when the run before them was as
 // long: a program that advances a small cavity a few steps at a time spends most of such a call
 // in the launches (10 steps and the fields at 24^3: 81 -> 77 us a call).
 constexpr int64_t kRunMin = 4, kRunMax = 128;
 template <typename S>
 static int run_part(lbm_ctx* c, const ParamsOf<S>& p, int64_t n) {
-    const bool again = n >= kRunMin && n <= kRunMax && n == c->last_run;
+    const bool again = n >= kRunMin && n <= kRunMax && n == c->last_run && !capturing(c->stream);
     c->last_run = n;
     cudaGraphExec_t g = nullptr;
     if (again) {

@@ -23,3 +23,31 @@ def test_runs_of_steps_equal_one_call(precision, interval):
         assert np.array_equal(x, y)
     a.close()
     b.close()
+
+
+def test_runs_recorded_into_the_callers_graph():
+    import torch
+    import paper_1710_04751_gb300 as lbm
+    kw = dict(Ra=2e3, precision=lbm.FP32, noise_amp=0.1, residual_interval=0)
+    st = torch.cuda.Stream()
+    a, b = lbm.LBM((12, 9, 7), 15, stream=st, **kw), lbm.LBM((12, 9, 7), 15, **kw)
+    for _ in range(3):
+        a.step(8)  # by now a graph of the library's own
+    a.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        a.step(8)
+        a.step(6)
+        a.step(6)
+    with torch.cuda.stream(st):
+        g.replay()
+        g.replay()
+    b.step(24 + 2 * 20)
+    for x, y in zip(a.get_populations(), b.get_populations()):
+        assert np.array_equal(x, y)
+    a.step(8)
+    b.step(8)
+    for x, y in zip(a.get_populations(), b.get_populations()):
+        assert np.array_equal(x, y)
+    a.close()
+    b.close()
