@@ -28,10 +28,10 @@ struct DevParams {
 
 // Whether `bytes` of state, one copy of what a step works through, fit into the L2 cache next to
 // the copy being written, given that the loads let go of what they read (load_pop in
-// node.cuh).  Measured per step with / without, FP32: 72^3 D3Q15 (45 MB) 17.3 / 17.8 us, 80^3
-// (61 MB) 20.7 / 23.6, 91^3 D3Q7 (66 MB) 19.3 / 23.8, 88^3 (82 MB) 27.0 / 28.8, 100^3 D3Q7
-// (88 MB) 29.0 / 31.7, 92^3 (93 MB) 32.8 / 33.8; 96^3 (106 MB) 37.8 / 37.1, 128^3 (252 MB)
-// 81.2 / 78.6.  (GB300's L2 holds 128 MB.)
+// node.cuh).  Measured per step with / without, FP32: 64^3 D3Q15 (31 MB) 8.5 / 8.5 us, 80^3
+// (61 MB) 17.6 / 19.9, 91^3 D3Q7 (66 MB) 19.2 / 23.6, 90^3 (87 MB) 27.1 / 30.6, 92^3 (93 MB)
+// 29.8 / 31.4; 104^3 D3Q7 (99 MB) 33.0 / 32.1, 96^3 (106 MB) 33.2 / 34.0, 128^3 (252 MB)
+// 80.7 / 75.6.  (GB300's L2 holds 128 MB.)
 inline bool state_fits_l2(int64_t bytes) { return bytes <= 96000000; }
 
 // Host-side view of one context's device buffers for the launchers.

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(128, (cavity_min_blocks<S, Q>() - (IMPOSE && c
 // Pair kernel of the 16-bit forms: one thread per pair of nodes (2t, 2t+1) of an x-row
 // (blockIdx.y = j, blockIdx.z = k), nx even.  Rows away from the y and z walls take the
 // packed pair update (pair.cuh); rows at a y or z wall update the two nodes one after
-// the other with the general pull.
+// the other with the one-node update.
 // ---------------------------------------------------------------------------------
 constexpr int kPairThreads = 64;
 
@@ -96,12 +96,12 @@ constexpr int kPairThreads = 64;
 #ifndef LBM_PAIR_MIN_BLOCKS_Q7
 #define LBM_PAIR_MIN_BLOCKS_Q7 8
 #endif
-// The unit-rate pair update (fewer live values): D3Q15 measured best at 8 blocks of 64
-// (128 registers; 10 and 14 blocks were 4% and 7% slower at 128^3), D3Q7 at 14 (72
-// registers; 10% faster than 8 at 128^3 and 256^3).  FP16 D3Q15 with every load issued
-// ahead of the arithmetic (pair_node_unit_early) needs 106 registers, and at 10 blocks it
-// is 4.5% faster than the compiler's order at 8 (68.4 against 71.6 us at 128^3, 426 against
-// 443 us at 256^3); BF16 measured 2% slower that way and keeps the compiler's order.
+// The unit-rate pair update (fewer live values): BF16 D3Q15 measured best at 8 blocks of 64 (128
+// registers; 54.9 us at 128^3, 55.6 at 10 blocks), D3Q7 at 14 (72 registers; FP16 38.3 us, 39.0 at
+// 12).  FP16 D3Q15 issues every load ahead of the arithmetic (pair_node_unit_early), at 10 blocks:
+// 54.8 us at 128^3 (8 blocks 55.3, 12 with spills 63.0) and 404 at 256^3.  BF16 that way is 2-3%
+// faster at 128^3 and 256^3 (53.4, 397 against 405) and 5% slower at 64^3 (8.7 against 8.3), FP16
+// D3Q7 4% slower at 128^3: they keep the compiler's order.
 #ifndef LBM_PAIR_UNIT_MIN_BLOCKS_Q15
 #define LBM_PAIR_UNIT_MIN_BLOCKS_Q15 8
 #endif
@@ -263,9 +263,10 @@ bool cavity_kernel_fits(const DevParams<real>& p) {
 
 // Threads of a cavity-kernel block, along x.  FP64: one warp.  The two FP64 lanes per clock and
 // SM bound the kernel, so what counts is that every SM gets the same number of working warps:
-// at 32^3 a block of 128 threads per row held one working warp and the registers of four.
-// 42 -> 28 us a step at 32^3.  Single precision: the lanes of a row's last block that are left
-// idle cost nothing measurable (rows of 24, 64, 91 packed without gaps: 0.98-1.0x).
+// at 32^3 a block of 128 threads per row holds one working warp and the registers of four.  33.4
+// against 23.4 us a step at 32^3, 108 against 100 at 48^3.  FP32: blocks of 32, 64 or 96 threads,
+// several rows to a block, or rows packed without gaps are within 3% at some sizes and up to 30%
+// slower at others (D3Q15 64^3 8.8 / 8.2 / 8.6 us against 8.5, 80^3 20.0 / 21.9 / 17.5 against 17.6).
 template <typename S>
 constexpr int cavity_threads() {
     return sizeof(typename Storage<S>::real) == 8 ? 32 : 128;
