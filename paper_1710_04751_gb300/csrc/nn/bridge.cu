@@ -90,8 +90,9 @@ cudaError_t launch_resample(const float* pred, int m, const lbm_grid& g, double 
                             cudaStream_t st) {
     const size_t smem = (size_t)4 * m * sizeof(double);
     if (smem > 40 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(resample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)std::min<size_t>(smem, 220 * 1024));
+        // one value for every caller: two threads may launch with different m
+        const cudaError_t e =
+            cudaFuncSetAttribute(resample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         if (e != cudaSuccess) return e;
     }
     const int64_t chunks = ((int64_t)g.ny * g.nz + kResampleRows - 1) / kResampleRows;
