@@ -417,18 +417,16 @@ static int run_part(lbm_ctx* c, const ParamsOf<S>& p, int64_t n) {
     c->last_run = n;
     cudaGraphExec_t g = nullptr;
     if (again) {
-        if (c->run_len != n) {
-            if (c->run_graph[0] || c->run_graph[1]) {  // the last run of the old length may still be at work
-                const int rc = wait_stream(c);
-                if (rc != LBM_OK) return rc;
-            }
+        // the graphs of another length go once nothing is at work that may be a launch of theirs
+        if (c->run_len != n && cudaStreamQuery(c->stream) == cudaSuccess) {
             for (cudaGraphExec_t& old : c->run_graph) {
                 if (old) cudaGraphExecDestroy(old);
                 old = nullptr;
             }
             c->run_len = n;
         }
-        g = step_graph<S>(c, p, c->cur, n, false, &c->run_graph[c->cur]);
+        if (c->run_len == n) g = step_graph<S>(c, p, c->cur, n, false, &c->run_graph[c->cur]);
+        else cudaGetLastError();  // not idle: no error of ours
     }
     if (g) {
         CUDA_OR_FAIL(c, cudaGraphLaunch(g, c->stream));

@@ -51,3 +51,21 @@ def test_runs_recorded_into_the_callers_graph():
         assert np.array_equal(x, y)
     a.close()
     b.close()
+
+
+def test_runs_of_a_new_length_do_not_wait_for_the_old_ones():
+    import paper_1710_04751_gb300 as lbm
+    kw = dict(Ra=2e3, precision=lbm.FP32, noise_amp=0.1, residual_interval=0)
+    a, b = lbm.LBM((96, 96, 96), 15, **kw), lbm.LBM((96, 96, 96), 15, **kw)
+    runs = [100, 100, 100, 90, 90, 80, 80, 80, 100, 100]
+    a.set_timeout(1e-9)  # any wait for the GPU would run out
+    for n in runs:
+        a.step(n)
+    a.set_timeout(600.0)
+    a.synchronize()
+    a.step(80)
+    b.step(sum(runs) + 80)
+    for x, y in zip(a.get_populations(), b.get_populations()):
+        assert np.array_equal(x, y)
+    a.close()
+    b.close()
