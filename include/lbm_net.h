@@ -45,8 +45,8 @@ int lbm_nn_gemm_bf16(const void* A, int64_t lda, const void* B, int64_t ldb, voi
  * [batch n^3][cout]: LBM_CONV_BIAS_RELU_BF16 writes BF16 max(y + bias, 0) (bias: device
  * FP32 [cout]), LBM_CONV_F32 writes the FP32 sums y.  Each K block's operand tile is one
  * TMA box of X shifted by the tap, zero-filled outside the grid: no im2col matrix.  cin a
- * multiple of 32, n a power of two in 2..256, cout <= 256, 16-byte aligned bases; else
- * LBM_EINVAL.  Waits for `cuda_stream` (bounded); LBM_ETIMEOUT as lbm_nn_gemm_bf16. */
+ * multiple of 32, n a power of two in 2..256, batch n^3 <= 2^31 - 128, cout <= 256, 16-byte
+ * aligned bases; else LBM_EINVAL.  Waits for `cuda_stream` (bounded); LBM_ETIMEOUT as lbm_nn_gemm_bf16. */
 enum { LBM_CONV_BIAS_RELU_BF16 = 0, LBM_CONV_F32 = 1 };
 
 /* dWT[r][co] += sum over voxels v of X[v + shift(tap)][ci] dZ[v][co], r = tap cin + ci (the

@@ -128,10 +128,10 @@ extern "C" int lbm_nn_conv3d_bf16(const void* X, int batch, int n, int cin, cons
         return record_error(nullptr, LBM_EINVAL, "NULL operand%s");
     if (mode != LBM_CONV_BIAS_RELU_BF16 && mode != LBM_CONV_F32)
         return record_error(nullptr, LBM_EINVAL, "invalid convolution mode%s");
-    if (!nn::conv_implicit_supported(n, cin, cout) || batch < 1)
+    if (!nn::conv_implicit_supported(n, cin, cout) || !nn::conv_rows_supported(batch, n))
         return record_error(nullptr, LBM_EINVAL,
                             "implicit convolution needs cin a multiple of 32, n a power of two in 2..256, "
-                            "1 <= cout <= 256 and batch >= 1%s");
+                            "1 <= cout <= 256, batch >= 1 and batch n^3 <= 2^31 - 128%s");
     ErrorWord* err = error_word();
     if (!err) return record_error(nullptr, LBM_ECUDA, "no CUDA device%s");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);

@@ -1073,6 +1073,11 @@ cudaError_t launch_wgrad(const CUtensorMap& tx, const CUtensorMap& tb, const Wgr
 
 }  // namespace
 
+// Rows are 32-bit in the kernels, up to the end of the last 128-row tile.
+bool conv_rows_supported(int B, int n) {
+    return B >= 1 && (int64_t)B * n * n * n <= (int64_t(1) << 31) - CBM;
+}
+
 bool conv_implicit_supported(int n, int cin, int cout) {
     return cin % 32 == 0 && n >= 2 && n <= 256 && (n & (n - 1)) == 0 && cout >= 1 && cout <= 256;
 }
@@ -1080,7 +1085,7 @@ bool conv_implicit_supported(int n, int cin, int cout) {
 cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const __nv_bfloat16* W,
                           long long ldw, int cout, const float* bias, void* out, int mode, int* err,
                           cudaStream_t st) {
-    if (!conv_implicit_supported(n, cin, cout) || B < 1 || ((uintptr_t)X & 15) || ((uintptr_t)W & 15) ||
+    if (!conv_implicit_supported(n, cin, cout) || !conv_rows_supported(B, n) || ((uintptr_t)X & 15) || ((uintptr_t)W & 15) ||
         (ldw % 8) || ldw < 27LL * cin || (mode == CONV_BIAS_RELU_BF16 && !bias) ||
         (mode != CONV_BIAS_RELU_BF16 && mode != CONV_F32))
         return cudaErrorInvalidValue;

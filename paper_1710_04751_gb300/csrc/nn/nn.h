@@ -30,9 +30,11 @@ size_t gemm_splitk_floats(int M, long long ldc, int K, int splits);
 // 3x3x3 convolution with zero padding as an implicit GEMM (conv.cu): X [B][n][n][n][cin]
 // BF16 channels last, W [cout][ldw] BF16 (K index tap * cin + ci), out [B n^3][cout]:
 // CONV_BIAS_RELU_BF16 writes bf16(max(y + bias, 0)), CONV_F32 writes y.  Needs
-// conv_implicit_supported (cin a multiple of 32, n a power of two); 16-byte aligned bases.
+// conv_implicit_supported (cin a multiple of 32, n a power of two) and conv_rows_supported
+// (B n^3 <= 2^31 - 128); 16-byte aligned bases.
 enum { CONV_BIAS_RELU_BF16 = 0, CONV_F32 = 1 };
 bool conv_implicit_supported(int n, int cin, int cout);
+bool conv_rows_supported(int B, int n);
 cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const __nv_bfloat16* W,
                           long long ldw, int cout, const float* bias, void* out, int mode, int* err,
                           cudaStream_t st);
