@@ -46,7 +46,8 @@ int lbm_nn_gemm_bf16(const void* A, int64_t lda, const void* B, int64_t ldb, voi
  * FP32 [cout]), LBM_CONV_F32 writes the FP32 sums y.  Each K block's operand tile is one
  * TMA box of X shifted by the tap, zero-filled outside the grid: no im2col matrix.  cin a
  * multiple of 32, n a power of two in 2..256, batch n^3 <= 2^31 - 128, cout <= 256, 16-byte
- * aligned bases; else LBM_EINVAL.  Waits for `cuda_stream` (bounded); LBM_ETIMEOUT as lbm_nn_gemm_bf16. */
+ * aligned bases (bias, and out where cout is not a multiple of 8: aligned to their elements);
+ * else LBM_EINVAL.  Waits for `cuda_stream` (bounded); LBM_ETIMEOUT as lbm_nn_gemm_bf16. */
 enum { LBM_CONV_BIAS_RELU_BF16 = 0, LBM_CONV_F32 = 1 };
 
 /* dWT[r][co] += sum over voxels v of X[v + shift(tap)][ci] dZ[v][co], r = tap cin + ci (the
@@ -59,7 +60,7 @@ enum { LBM_CONV_BIAS_RELU_BF16 = 0, LBM_CONV_F32 = 1 };
  * splits' partial tiles go to `ws` (device FP32 scratch of at least splits Kp cout values)
  * and are added to dWT in split order, so the result is the same on every run.  n a power
  * of two in 2..256, cin a multiple of 32, cout a multiple of 8 in 8..256, 16-byte aligned
- * bases; else LBM_EINVAL.  Waits for `cuda_stream` (bounded); LBM_ETIMEOUT as
+ * bases (dWT, and ws where cout is 8: aligned to their elements); else LBM_EINVAL.  Waits for `cuda_stream` (bounded); LBM_ETIMEOUT as
  * lbm_nn_gemm_bf16. */
 int lbm_nn_conv3d_wgrad_bf16(const void* X, int batch, int n, int cin, const void* dZ, int cout, int Kp,
                              float* ws, int64_t ws_floats, int splits, float* dWT, void* cuda_stream);

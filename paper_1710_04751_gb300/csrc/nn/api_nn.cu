@@ -108,6 +108,8 @@ extern "C" int lbm_nn_conv3d_wgrad_bf16(const void* X, int batch, int n, int cin
         return record_error(nullptr, LBM_EINVAL,
                             "implicit weight gradient needs n a power of two in 2..256, cin a multiple of 32, "
                             "cout a multiple of 8 in 8..256, Kp >= 27 cin and splits >= 1%s");
+    if (!nn::conv_wgrad_bases_supported(X, dZ, ws, dWT, cout))
+        return record_error(nullptr, LBM_EINVAL, "a base of the weight gradient is not aligned%s");
     ErrorWord* err = error_word();
     if (!err) return record_error(nullptr, LBM_ECUDA, "no CUDA device%s");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
@@ -132,6 +134,8 @@ extern "C" int lbm_nn_conv3d_bf16(const void* X, int batch, int n, int cin, cons
         return record_error(nullptr, LBM_EINVAL,
                             "implicit convolution needs cin a multiple of 32, n a power of two in 2..256, "
                             "1 <= cout <= 256, batch >= 1 and batch n^3 <= 2^31 - 128%s");
+    if (!nn::conv_bases_supported(X, W, bias, out, cout, mode == LBM_CONV_F32 ? nn::CONV_F32 : nn::CONV_BIAS_RELU_BF16))
+        return record_error(nullptr, LBM_EINVAL, "a base of the convolution is not aligned%s");
     ErrorWord* err = error_word();
     if (!err) return record_error(nullptr, LBM_ECUDA, "no CUDA device%s");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);

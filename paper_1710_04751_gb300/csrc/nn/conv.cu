@@ -1078,6 +1078,13 @@ bool conv_rows_supported(int B, int n) {
     return B >= 1 && (int64_t)B * n * n * n <= (int64_t(1) << 31) - CBM;
 }
 
+// Operands that TMA reads start on 16 bytes, and so does an output written in 16-byte pieces
+// (conv_store16, x3_store16: rows of a multiple of 8 values); else it is aligned to its elements.
+bool conv_bases_supported(const void* X, const void* W, const float* bias, const void* out, int cout, int mode) {
+    const uintptr_t o = cout % 8 == 0 ? 15 : mode == CONV_F32 ? 3 : 1, b = mode == CONV_F32 ? 0 : 3;
+    return !((uintptr_t)X & 15) && !((uintptr_t)W & 15) && !((uintptr_t)bias & b) && !((uintptr_t)out & o);
+}
+
 bool conv_implicit_supported(int n, int cin, int cout) {
     return cin % 32 == 0 && n >= 2 && n <= 256 && (n & (n - 1)) == 0 && cout >= 1 && cout <= 256;
 }
@@ -1085,8 +1092,8 @@ bool conv_implicit_supported(int n, int cin, int cout) {
 cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const __nv_bfloat16* W,
                           long long ldw, int cout, const float* bias, void* out, int mode, int* err,
                           cudaStream_t st) {
-    if (!conv_implicit_supported(n, cin, cout) || !conv_rows_supported(B, n) || ((uintptr_t)X & 15) || ((uintptr_t)W & 15) ||
-        (ldw % 8) || ldw < 27LL * cin || (mode == CONV_BIAS_RELU_BF16 && !bias) ||
+    if (!conv_implicit_supported(n, cin, cout) || !conv_rows_supported(B, n) ||
+        !conv_bases_supported(X, W, bias, out, cout, mode) || (ldw % 8) || ldw < 27LL * cin || (mode == CONV_BIAS_RELU_BF16 && !bias) ||
         (mode != CONV_BIAS_RELU_BF16 && mode != CONV_F32))
         return cudaErrorInvalidValue;
     const int bkc = cin % 64 == 0 ? 64 : 32;
@@ -1190,11 +1197,18 @@ bool conv_wgrad_implicit_supported(int B, int n, int cin, int cout) {
            cout % 8 == 0 && B >= 1 && M < (int64_t(1) << 31) - 64;
 }
 
+// As conv_bases_supported; the slices of ws are written in 16-byte pieces but for the one-tap form
+// of 8 output channels.
+bool conv_wgrad_bases_supported(const void* X, const void* dZ, const float* ws, const float* dWT, int cout) {
+    return !((uintptr_t)X & 15) && !((uintptr_t)dZ & 15) && !((uintptr_t)ws & (cout > 8 ? 15 : 3)) &&
+           !((uintptr_t)dWT & 3);
+}
+
 cudaError_t conv_wgrad_implicit(const __nv_bfloat16* X, int B, int n, int cin, const __nv_bfloat16* dZ, int cout,
                                 int Kp, float* ws, size_t ws_floats, int splits, float* dWT, int accumulate,
                                 int* err, cudaStream_t st) {
-    if (!conv_wgrad_implicit_supported(B, n, cin, cout) || Kp < 27 * cin || splits < 1 || ((uintptr_t)X & 15) ||
-        ((uintptr_t)dZ & 15))
+    if (!conv_wgrad_implicit_supported(B, n, cin, cout) || Kp < 27 * cin || splits < 1 ||
+        !conv_wgrad_bases_supported(X, dZ, ws, dWT, cout))
         return cudaErrorInvalidValue;
     const int64_t M = (int64_t)B * n * n * n;
     const int kblocks = (int)((M + 63) / 64);
@@ -1206,7 +1220,7 @@ cudaError_t conv_wgrad_implicit(const __nv_bfloat16* X, int B, int n, int cin, c
     // 64^3 batch 2, 96 -> 32 channels 286 / 163 and 32 -> 32 136 / 101, 32^3 batch 2, 192 -> 64
     // 117 / 101; below that its long ramp shows: 32^3, 64 -> 64 79 / 82, 16^3 batch 4, 64 -> 48
     // 64 / 75.  More than 64 output channels fill the one-tap form's MMAs.
-    if (n >= 16 && cout <= 64 && M * cin >= (int64_t(1) << 23)) {
+    if (n >= 16 && cout <= 64 && M * cin >= (int64_t(1) << 23) && !((uintptr_t)ws & 15)) {
         int slices = 0;
         const cudaError_t e = launch_wgrad9(X, B, n, cin, dZ, cout, Kp, ws, used, &slices, err, st);
         if (e != cudaSuccess) return e;

@@ -31,10 +31,11 @@ size_t gemm_splitk_floats(int M, long long ldc, int K, int splits);
 // BF16 channels last, W [cout][ldw] BF16 (K index tap * cin + ci), out [B n^3][cout]:
 // CONV_BIAS_RELU_BF16 writes bf16(max(y + bias, 0)), CONV_F32 writes y.  Needs
 // conv_implicit_supported (cin a multiple of 32, n a power of two) and conv_rows_supported
-// (B n^3 <= 2^31 - 128); 16-byte aligned bases.
+// (B n^3 <= 2^31 - 128) and conv_bases_supported (aligned bases).
 enum { CONV_BIAS_RELU_BF16 = 0, CONV_F32 = 1 };
 bool conv_implicit_supported(int n, int cin, int cout);
 bool conv_rows_supported(int B, int n);
+bool conv_bases_supported(const void* X, const void* W, const float* bias, const void* out, int cout, int mode);
 cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const __nv_bfloat16* W,
                           long long ldw, int cout, const float* bias, void* out, int mode, int* err,
                           cudaStream_t st);
@@ -62,6 +63,7 @@ cudaError_t im2colT(const __nv_bfloat16* X, int B, int n, int cin, int Kp, __nv_
 // in 2..256, cin a multiple of 32, cout a multiple of 8 up to 256; ws holds splits Kp cout
 // floats (the split partials, added to dWT in split order; accumulate == 0: dWT = the sum).
 bool conv_wgrad_implicit_supported(int B, int n, int cin, int cout);
+bool conv_wgrad_bases_supported(const void* X, const void* dZ, const float* ws, const float* dWT, int cout);
 cudaError_t conv_wgrad_implicit(const __nv_bfloat16* X, int B, int n, int cin, const __nv_bfloat16* dZ, int cout,
                                 int Kp, float* ws, size_t ws_floats, int splits, float* dWT, int accumulate,
                                 int* err, cudaStream_t st);
