@@ -23,6 +23,7 @@
 
 #include "nn.h"
 #include "tc.cuh"
+#include "wgrad_plan.h"
 
 namespace lbm {
 namespace nn {
@@ -1140,28 +1141,13 @@ cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const _
     return bkc == 64 ? launch_conv_bkc<64>(tx, tw, a, BN, st) : launch_conv_bkc<32>(tx, tw, a, BN, st);
 }
 
-// The nine-tap weight gradient: the slices (at most max_slices) and whether CTAs go in pairs.
-// The tensor core's FP32 accumulation truncates, so the length of its chains shows in the
-// result: about 7e-10 of relative error per voxel of a chain.  A chain may be up to 1.15 times
-// as long as max_slices make it; two chains of half the length may take its place up to
-// kPairChain voxels, beyond which that would move a result by 2e-5.  Among these the choice
-// that leaves the least work to the busiest SM.
-constexpr int kPairChain = 38400;
+// The nine-tap weight gradient into *slices <= max_slices slices of ws (plan_wgrad9).
 cudaError_t launch_wgrad9(const __nv_bfloat16* X, int B, int n, int cin, const __nv_bfloat16* dZ, int cout, int Kp,
                           float* ws, int max_slices, int* slices, int* err, cudaStream_t st) {
     const int total = (int)((int64_t)B * n * n * n / 64);
-    const int mtiles = (3 * (cin / 32) + 3) / 4, ntiles = (cout + 31) / 32, tiles = mtiles * ntiles;
-    max_slices = std::min(max_slices, total);
-    int best_s = max_slices, best_c = 1;
-    int64_t best = INT64_MAX;
-    for (int c = 1; c <= ((int64_t)total * 64 <= (int64_t)kPairChain * max_slices ? 2 : 1); ++c)
-        for (int s = max_slices; s >= 1 && 100 * max_slices <= 115 * s; --s) {
-            const int64_t waves = ((int64_t)tiles * s * c + kSMs - 1) / kSMs;
-            const int64_t t = waves * ((total + s * c - 1) / (s * c) + 8);  // 8: prologue and drain
-            if (t < best) best = t, best_s = s, best_c = c;
-        }
-    const int per = (total + best_s * best_c - 1) / (best_s * best_c);
-    *slices = (total + per * best_c - 1) / (per * best_c);  // every slice has work in its first CTA
+    const int mtiles = (3 * (cin / 32) + 3) / 4, ntiles = (cout + 31) / 32;
+    const Wgrad9Plan plan = plan_wgrad9(total, cin, cout, max_slices);
+    *slices = plan.slices;
     constexpr int smem = 1024 + W9_RING + 256;
     const auto kernel = n == 16 ? conv_wgrad9_kernel<4> : n == 32 ? conv_wgrad9_kernel<2> : conv_wgrad9_kernel<1>;
     static std::once_flag once;
@@ -1175,19 +1161,19 @@ cudaError_t launch_wgrad9(const __nv_bfloat16* X, int B, int n, int cin, const _
     CUtensorMap tx, tz;
     if (!make_x_map(&tx, X, B, n, cin, 32, bx, RB, 1, 1) || !make_x_map(&tz, dZ, B, n, cout, 32, bx, 1, 1, 1))
         return cudaErrorInvalidValue;
-    const Wgrad9Args a{cout, cin, n, segs, n / RB, total, per, Kp, best_c == 2, ws, err};
+    const Wgrad9Args a{cout, cin, n, segs, n / RB, total, plan.per, Kp, plan.ctas == 2, ws, err};
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(*slices * best_c), (unsigned)mtiles, (unsigned)ntiles);
+    cfg.gridDim = dim3((unsigned)(plan.slices * plan.ctas), (unsigned)mtiles, (unsigned)ntiles);
     cfg.blockDim = dim3(128);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)best_c;
+    at[0].val.clusterDim.x = (unsigned)plan.ctas;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = best_c == 2 ? 1 : 0;
+    cfg.numAttrs = plan.ctas == 2 ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, tx, tz, a);
 }
 
