@@ -1202,11 +1202,9 @@ cudaError_t conv_wgrad_implicit(const __nv_bfloat16* X, int B, int n, int cin, c
     const int used = (kblocks + per - 1) / per;
     const int mtiles = (Kp + CBM - 1) / CBM;
     if ((size_t)used * Kp * cout > ws_floats) return cudaErrorInvalidValue;
-    // The nine-tap form where it measured faster (calls with the host wait, us, one-tap / nine-tap):
-    // 64^3 batch 2, 96 -> 32 channels 286 / 163 and 32 -> 32 136 / 101, 32^3 batch 2, 192 -> 64
-    // 117 / 101; below that its long ramp shows: 32^3, 64 -> 64 79 / 82, 16^3 batch 4, 64 -> 48
-    // 64 / 75.  More than 64 output channels fill the one-tap form's MMAs.
-    if (n >= 16 && cout <= 64 && M * cin >= (int64_t(1) << 23) && !((uintptr_t)ws & 15)) {
+    // The nine-tap form where it has less to do on the busiest SM (nine_taps_pay).  More than 64 output
+    // channels fill the one-tap form's MMAs.
+    if (n >= 16 && cout <= 64 && !((uintptr_t)ws & 15) && nine_taps_pay(M, cin, cout, Kp, used, per)) {
         int slices = 0;
         const cudaError_t e = launch_wgrad9(X, B, n, cin, dZ, cout, Kp, ws, used, &slices, err, st);
         if (e != cudaSuccess) return e;

@@ -47,7 +47,8 @@ def test_convolution_of_whole_numbers(B, n, cin, cout):
 
 WGRAD = [(3, 2, 32, 8, 1), (2, 8, 64, 48, 3), (4, 16, 64, 48, 5), (16, 16, 128, 64, 5), (17, 16, 128, 8, 3), (2, 32, 128, 40, 3),
          (3, 32, 96, 64, 7), (1, 32, 256, 24, 1), (2, 32, 64, 128, 9), (1, 64, 32, 24, 4), (2, 64, 96, 32, 14), (1, 64, 96, 48, 11),
-         (1, 64, 32, 32, 43), (1, 128, 32, 8, 9), (1, 128, 32, 32, 43), (1, 256, 32, 8, 8), (1, 256, 32, 32, 43)]
+         (1, 64, 32, 32, 43), (1, 128, 32, 8, 9), (1, 128, 32, 32, 43), (1, 256, 32, 8, 8), (1, 256, 32, 32, 43), (16, 16, 128, 64, 26), (3, 32, 96, 64, 14), (1, 64, 32, 24, 43),
+         (1, 64, 96, 48, 14), (1, 128, 32, 8, 43), (1, 256, 32, 8, 43)]
 
 
 @pytest.mark.parametrize("B,n,cin,cout,splits", WGRAD)
