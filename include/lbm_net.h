@@ -161,7 +161,9 @@ int lbm_net_targets(lbm_ctx* ctx, float* out);
  * grid covering the cavity, resampled trilinearly onto the context's grid (identity
  * when m equals it), scaled back (u = p U0, T = p / 2), and set as equilibria with
  * rho = 1 followed by `iterations` rounds of the consistent initialisation
- * (lbm_init_fields). */
+ * (lbm_init_fields).  With rounds, and always for the 16-bit forms, it allocates device scratch
+ * that it frees before it returns: at most 32 bytes a node, beyond the context's arena
+ * (LBM_ENOMEM if there is none). */
 int lbm_net_warm_start(lbm_ctx* ctx, const float* pred, int m, int iterations);
 
 #ifdef __cplusplus

@@ -723,38 +723,33 @@ extern "C" int lbm_set_fields(lbm_ctx* c, const double* rho, const double* ux, c
     return lbm_init_fields(c, rho, ux, uy, uz, T, 0);
 }
 
-bool lbm::rounds_fused(lbm_ctx* c) {
+bool lbm::rounds_fused(const lbm_ctx* c) {
     return with_storage(c->precision, [&](auto tag) {
         using S = decltype(tag);
-        using real = typename Storage<S>::real;
-        if (!step_imposable<S>(c->dev, dev_params<real>(c))) return 0;
-        if (!c->imposed && cudaMalloc(&c->imposed, (size_t)4 * c->ncell * sizeof(real)) != cudaSuccess) {
-            cudaGetLastError();  // no room: the rounds run as two kernels each
-            c->imposed = nullptr;
-        }
-        return (int)(c->imposed != nullptr);
+        return (int)step_imposable<S>(c->dev, dev_params<typename Storage<S>::real>(c));
     });
 }
 
-extern "C" int lbm_init_fields(lbm_ctx* c, const double* rho, const double* ux, const double* uy,
-                               const double* uz, const double* T, int iterations) {
-    if (!c || !ux || !uy || !uz || !T || iterations < 0)
-        return fail(c, LBM_EINVAL, "NULL argument or negative iterations%s");
-    DeviceGuard gd(c->device);
+size_t lbm::packed_bytes(const lbm_ctx* c) { return (size_t)4 * c->ncell * compute_bytes(c->precision); }
+
+int lbm::init_fields(lbm_ctx* c, const double* rho, const double* ux, const double* uy, const double* uz,
+                     const double* T, int iterations, void* packed) {
     int rc = with_storage(c->precision, [&](auto tag) {
         using S = decltype(tag);
-        const ParamsOf<S> p = dev_params<typename Storage<S>::real>(c);
+        using real = typename Storage<S>::real;
+        const ParamsOf<S> p = dev_params<real>(c);
         CUDA_OR_FAIL(c, launch_set_fields<S>(c->dev, c->cur, p, rho, ux, uy, uz, T, c->stream));
         const int rounds = iterations + (iterations & 1);  // even: the state stays in its buffer
-        using real = typename Storage<S>::real;
-        const bool fused = rounds > 0 && rounds_fused(c);
-        if (fused) {  // the fields are read here for the last time
-            real* w = static_cast<real*>(c->imposed);
-            CUDA_OR_FAIL(c, launch_pack_imposed<real>(ux, uy, uz, T, c->ncell, w, c->stream));
-            for (int it = 0; it < rounds; ++it, c->cur ^= 1)
-                CUDA_OR_FAIL(c, launch_step_imposed<S>(c->dev, c->cur, p, w, c->stream));
-        }
-        for (int it = 0; it < rounds && !fused; ++it) {
+        const bool fused = step_imposable<S>(c->dev, p);
+        if (fused && packed)
+            CUDA_OR_FAIL(c, launch_pack_imposed<real>(ux, uy, uz, T, c->ncell, static_cast<real*>(packed), c->stream));
+        const ImposedFields fields{ux, uy, uz, T, packed};
+        for (int it = 0; it < rounds; ++it) {
+            if (fused) {
+                CUDA_OR_FAIL(c, launch_step_imposed<S>(c->dev, c->cur, p, fields, c->stream));
+                c->cur ^= 1;
+                continue;
+            }
             CUDA_OR_FAIL(c, launch_step<S>(c->dev, c->cur, p, c->stream));
             c->cur ^= 1;
             CUDA_OR_FAIL(c, launch_reimpose<S>(c->dev, c->cur, p, ux, uy, uz, T, c->stream));
@@ -765,6 +760,14 @@ extern "C" int lbm_init_fields(lbm_ctx* c, const double* rho, const double* ux, 
     if (rc != LBM_OK) return rc;
     c->last_residual = -1.0;
     return wait_stream(c);
+}
+
+extern "C" int lbm_init_fields(lbm_ctx* c, const double* rho, const double* ux, const double* uy,
+                               const double* uz, const double* T, int iterations) {
+    if (!c || !ux || !uy || !uz || !T || iterations < 0)
+        return fail(c, LBM_EINVAL, "NULL argument or negative iterations%s");
+    DeviceGuard gd(c->device);
+    return init_fields(c, rho, ux, uy, uz, T, iterations, nullptr);
 }
 
 // ---------------------------------------------------------------------------------
@@ -909,7 +912,6 @@ void lbm::destroy_context(lbm_ctx* c) {
         for (cudaGraphExec_t* g : {&c->step_graph[0], &c->step_graph[1], &c->run_graph[0], &c->run_graph[1]})
             if (*g) cudaGraphExecDestroy(*g);
         if (c->capture) cudaStreamDestroy(c->capture);
-        if (c->imposed) cudaFree(c->imposed);
         if (c->own_arena && c->arena) cudaFree(c->arena);
         if (c->host_bits) cudaFreeHost(c->host_bits);
     }

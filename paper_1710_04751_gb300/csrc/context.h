@@ -61,9 +61,6 @@ struct lbm_ctx {
     bool graphs_failed = false;  // capture not possible here: launch the steps one by one
     // state_fits_l2 of everything a step goes through: this context, the batch or all slabs
     bool in_l2 = false;
-    // (u_x, u_y, u_z, T) of lbm_init_fields in the arithmetic type, for its rounds of one step
-    // and a reimposition; allocated at the first such call, freed with the context
-    void* imposed = nullptr;
     int64_t cell0 = 0;  // global index of cell 0 (slabs of a larger grid), for the initial noise
 };
 
@@ -104,9 +101,15 @@ int transfer_cells(lbm_ctx* c, double* f, double* g, const double* fin, const do
                    int64_t first, int64_t count, int64_t hstride);
 int transfer_done(lbm_ctx* c, bool uploaded);
 
-// Whether lbm_init_fields runs each of its rounds as one kernel on this context (and reads the
-// given fields only before the first); makes room for the packed fields at the first call.
-bool rounds_fused(lbm_ctx* c);
+// Whether lbm_init_fields runs each of its rounds as one kernel on this context, and the bytes of
+// its fields packed for that kernel.
+bool rounds_fused(const lbm_ctx* c);
+size_t packed_bytes(const lbm_ctx* c);
+
+// lbm_init_fields on checked arguments.  packed: NULL, or device scratch of packed_bytes for the
+// rounds: with rounds_fused, ux .. T are then read before the first round only.
+int init_fields(lbm_ctx* c, const double* rho, const double* ux, const double* uy, const double* uz,
+                const double* T, int iterations, void* packed);
 
 // lbm_fields for cells [first, first + count): outs[w] (rho, ux, uy, uz, T; NULL = skip)
 // receive count values each.

@@ -109,18 +109,24 @@ template <typename S>
 cudaError_t launch_reimpose(const DevState& s, int cur, const ParamsOf<S>& p, const double* ux,
                             const double* uy, const double* uz, const double* T, cudaStream_t st);
 
+// Device fields of ncell FP64 values each; packed: NULL, or the same as [ncell][4] = (u_x, u_y, u_z,
+// T) in the arithmetic type, aligned to a quadruple (launch_pack_imposed), which is then read instead.
+struct ImposedFields {
+    const double *ux, *uy, *uz, *T;
+    const void* packed;
+};
+
 // The step and the reimposition above in one kernel: the reimposition alone read and wrote the
 // whole state once more and ran four general collisions a node (205 us at 128^3, FP32, next to
 // the step's 75), while the step holds the departure from equilibrium in registers; together
-// 85 us a round.  FP32 and FP64 cavities at the paper's unit
-// higher-order rates (step_imposable), reading the state of buffer `cur`, writing the other.
-// imposed: [ncell][4] = (u_x, u_y, u_z, T) in the context's arithmetic type (pack_imposed),
-// aligned to a quadruple.
+// 85 us a round with the fields read as they are given, 80 packed, with the same result.  FP32 and
+// FP64 cavities at the paper's unit higher-order rates (step_imposable), reading the state of
+// buffer `cur`, writing the other.
 template <typename S>
 bool step_imposable(const DevState& s, const ParamsOf<S>& p);
 template <typename S>
-cudaError_t launch_step_imposed(const DevState& s, int cur, const ParamsOf<S>& p,
-                                const typename Storage<S>::real* imposed, cudaStream_t st);
+cudaError_t launch_step_imposed(const DevState& s, int cur, const ParamsOf<S>& p, const ImposedFields& imposed,
+                                cudaStream_t st);
 template <typename real>
 cudaError_t launch_pack_imposed(const double* ux, const double* uy, const double* uz, const double* T,
                                 int64_t n, real* out, cudaStream_t st);

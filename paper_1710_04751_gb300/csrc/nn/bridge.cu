@@ -21,7 +21,7 @@ namespace {
 // (y, z) is interpolated once into shared memory (4 m values), and every node adds one
 // interpolation in x with weights its thread keeps from row to row: about 30 operations a node
 // instead of 170.  A warm start 64^3 -> 128^3 with 50 rounds and the fields read back, with
-// the fused rounds (launch_step_imposed): 15.6 -> 4.6 ms.
+// the fused rounds (launch_step_imposed): 15.6 -> 4.5 ms.
 constexpr int kResampleThreads = 128, kResampleRows = 16;
 
 // Position of node i of n on an axis of m cells: cells lo and hi = lo + 1 with weights 1 - w
@@ -124,20 +124,26 @@ extern "C" int lbm_net_warm_start(lbm_ctx* c, const float* pred, int m, int iter
     if (!(c->params.U0 > 0)) return fail(c, LBM_EINVAL, "the context has no velocity scale U0%s");
     DeviceGuard g(c->device);
     const int64_t n = c->ncell;
-    // The FP64 fields go to the flow planes of the buffer the next step writes when nothing
-    // reads them after lbm_init_fields has (FP32 and FP64); else to memory of their own.
+    // The FP64 fields go to the flow planes of the buffer the next step writes when nothing reads them
+    // after the first round (FP32 and FP64), and the rounds take them packed from memory of the call's
+    // own (16 bytes a node in FP32, where the fields themselves take 32); else the fields go there.
+    // That memory is allocated and freed on each call (33 MB: 0.12 ms, half of it beside the resampling):
+    // kept, it would be device memory that no arena counts.
     const bool dev16 = c->precision == LBM_FP16_DEV || c->precision == LBM_BF16_DEV;
-    const bool lend = !dev16 && (iterations == 0 || rounds_fused(c));
-    double* own = nullptr;
+    const bool lend = iterations == 0 ? !dev16 : rounds_fused(c);
+    const size_t bytes = !lend ? (size_t)4 * n * sizeof(double) : iterations ? packed_bytes(c) : 0;
+    double* buf = static_cast<double*>(c->dev.F[c->cur ^ 1]);
+    void* own = nullptr;
+    cudaError_t e = lend ? launch_resample(pred, m, c->grid, c->params.U0, buf, n, c->stream) : cudaSuccess;
+    if (bytes && cudaMalloc(&own, bytes) != cudaSuccess)
+        return fail(c, LBM_ENOMEM, "cudaMalloc failed: %s", cudaGetErrorString(cudaGetLastError()));
     if (!lend) {
-        const cudaError_t e = cudaMalloc(&own, (size_t)4 * n * sizeof(double));
-        if (e != cudaSuccess) return fail(c, LBM_ENOMEM, "cudaMalloc failed: %s", cudaGetErrorString(e));
+        buf = static_cast<double*>(own);
+        e = launch_resample(pred, m, c->grid, c->params.U0, buf, n, c->stream);
     }
-    double* buf = lend ? static_cast<double*>(c->dev.F[c->cur ^ 1]) : own;
-    const cudaError_t e = launch_resample(pred, m, c->grid, c->params.U0, buf, n, c->stream);
     int rc = e == cudaSuccess
-                 ? lbm_init_fields(c, nullptr, buf, buf + n, buf + 2 * n, buf + 3 * n, iterations)
+                 ? init_fields(c, nullptr, buf, buf + n, buf + 2 * n, buf + 3 * n, iterations, lend ? own : nullptr)
                  : fail(c, LBM_ECUDA, "resampling failed: %s", cudaGetErrorString(e));
-    if (own) cudaFree(own);  // lbm_init_fields waited for the stream
+    if (own) cudaFree(own);  // init_fields waited for the stream
     return rc;
 }

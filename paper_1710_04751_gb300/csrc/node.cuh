@@ -165,15 +165,15 @@ __device__ __forceinline__ void pull_wall(const S* __restrict__ Fin, const S* __
 // only the low-order moments of the pulled populations.
 // seed: the node's rounding dither (dither_seed of its global index and the step) for
 // the stochastically rounded flow stores of the 16-bit forms; unused otherwise.
-// IMPOSE (unit rates, FP32 and FP64): the stored state is moved to the u and T of
-// imposed[c] = (u_x, u_y, u_z, T), keeping the node's departure from equilibrium.
+// IMPOSE (unit rates, FP32 and FP64): the stored state is moved to the u and T of `imposed`,
+// keeping the node's departure from equilibrium.
 template <typename S, int Q, bool UNIT = false, bool IMPOSE = false>
 __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15],
                                               typename Storage<S>::real (&g)[Q],
                                               S* __restrict__ Fout, S* __restrict__ Gout,
                                               float* __restrict__ Tout,
                                               const ParamsOf<S>& p, int64_t c, uint32_t seed = 0,
-                                              const typename Storage<S>::real* __restrict__ imposed = nullptr) {
+                                              const ImposedFields& imposed = ImposedFields{}) {
     using real = typename Storage<S>::real;
     using St = Storage<S>;
     const int64_t P = p.plane;
@@ -217,12 +217,17 @@ __device__ __forceinline__ void collide_store(typename Storage<S>::real (&f)[15]
         UPow<real> v;
         if constexpr (IMPOSE) {
             static_assert(!St::deviation, "the 16-bit forms impose in a pass of their own");
-            struct alignas(4 * sizeof(real)) Four {
-                real x, y, z, t;
-            };
-            const Four w = reinterpret_cast<const Four*>(imposed)[c];
-            Ts = w.t;
-            v = upow<real>(w.x, w.y, w.z);
+            if (imposed.packed) {
+                struct alignas(4 * sizeof(real)) Four {
+                    real x, y, z, t;
+                };
+                const Four w = static_cast<const Four*>(imposed.packed)[c];
+                Ts = w.t;
+                v = upow<real>(w.x, w.y, w.z);
+            } else {
+                Ts = (real)imposed.T[c];
+                v = upow<real>((real)imposed.ux[c], (real)imposed.uy[c], (real)imposed.uz[c]);
+            }
             flow_unit_imposed<real>(dm, Fx, Fy, Fz, r, inv_rho, u, v, D);
         } else {
             flow_unit<real>(dm, Fx, Fy, Fz, r, inv_rho, u, D);
@@ -293,7 +298,7 @@ __device__ __forceinline__ void cavity_node(const S* __restrict__ Fin, const S* 
                                             S* __restrict__ Gout, float* __restrict__ Tout,
                                             const ParamsOf<S>& p, int i, int j, int k,
                                             uint32_t step = 0,
-                                            const typename Storage<S>::real* __restrict__ imposed = nullptr) {
+                                            const ImposedFields& imposed = ImposedFields{}) {
     using real = typename Storage<S>::real;
     using St = Storage<S>;
     const int nx = p.nx;

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(128, (cavity_min_blocks<S, Q>() - (IMPOSE && c
                        const float* __restrict__ Tin, S* __restrict__ Fout,
                        S* __restrict__ Gout, float* __restrict__ Tout, ParamsOf<S> p,
                        const unsigned* __restrict__ ctr_in, unsigned* __restrict__ ctr_out,
-                       const typename Storage<S>::real* __restrict__ imposed) {
+                       ImposedFields imposed) {
     pdl_begin();
     const uint32_t step = step_of<S>(ctr_in, ctr_out);
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -272,11 +272,11 @@ constexpr int cavity_threads() {
     return sizeof(typename Storage<S>::real) == 8 ? 32 : 128;
 }
 
-// One step of a cavity at unit rates whose result is moved to the u and T of imposed
-// ([ncell][4] = u_x, u_y, u_z, T, aligned to a quadruple); only where step_imposable says so.
+// One step of a cavity at unit rates whose result is moved to the u and T of imposed; only where
+// step_imposable says so.
 template <typename S>
-cudaError_t launch_step_imposed_as(const DevState& s, int cur, const ParamsOf<S>& p,
-                                   const typename Storage<S>::real* imposed, cudaStream_t st) {
+cudaError_t launch_step_imposed_as(const DevState& s, int cur, const ParamsOf<S>& p, const ImposedFields& imposed,
+                                   cudaStream_t st) {
     const S* Fin = static_cast<const S*>(s.F[cur]);
     const S* Gin = static_cast<const S*>(s.G[cur]);
     S* Fout = static_cast<S*>(s.F[cur ^ 1]);
@@ -308,7 +308,7 @@ cudaError_t launch_step_as(const DevState& s, int cur, const ParamsOf<S>& p, cud
     if (cavity_kernel_fits(p)) {
         const int bx = cavity_threads<S>();
         const dim3 grid((p.nx + bx - 1) / bx, p.ny, p.nz);
-        const typename Storage<S>::real* none = nullptr;
+        const ImposedFields none{};
         if (s.Q == 15)
             return launch_pdl(step_cavity_kernel<S, 15, UNIT>, grid, dim3(bx), st, Fin, Gin, Tin, Fout, Gout,
                               Tout, p, ctr_in, ctr_out, none);

@@ -21,8 +21,8 @@ bool step_imposable(const DevState& s, const ParamsOf<S>& p) {
 }
 
 template <typename S>
-cudaError_t launch_step_imposed(const DevState& s, int cur, const ParamsOf<S>& p,
-                                const typename Storage<S>::real* imposed, cudaStream_t st) {
+cudaError_t launch_step_imposed(const DevState& s, int cur, const ParamsOf<S>& p, const ImposedFields& imposed,
+                                cudaStream_t st) {
     if constexpr (Storage<S>::deviation) return cudaErrorNotSupported;
     else return launch_step_imposed_as<S>(s, cur, p, imposed, st);
 }
@@ -30,7 +30,7 @@ cudaError_t launch_step_imposed(const DevState& s, int cur, const ParamsOf<S>& p
 #define LBM_INSTANTIATE_IMPOSED(S)                                                                  \
     template bool step_imposable<S>(const DevState&, const ParamsOf<S>&);                            \
     template cudaError_t launch_step_imposed<S>(const DevState&, int, const ParamsOf<S>&,            \
-                                                const Storage<S>::real*, cudaStream_t);
+                                                const ImposedFields&, cudaStream_t);
 LBM_INSTANTIATE_IMPOSED(double)
 LBM_INSTANTIATE_IMPOSED(float)
 LBM_INSTANTIATE_IMPOSED(__half)
