@@ -367,6 +367,17 @@ static cudaError_t enqueue_check(lbm_ctx* c, const ParamsOf<S>& p, int cur, int6
     return e != cudaSuccess ? e : launch_residual<S>(c->dev, cur, p, 1, st);
 }
 
+// The thread's calls are not held against a capture that it, or another thread, has under way on some
+// other stream: a query or a graph's instantiation here would end a capture in the global mode
+// (what torch.cuda.graph uses), while launches on a stream that is not captured do not.
+struct BesideCaptures {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    BesideCaptures(const BesideCaptures&) = delete;
+    BesideCaptures& operator=(const BesideCaptures&) = delete;
+};
+
 // A graph of n steps from buffer `cur`, and of the check of a whole residual interval, in *slot
 // (captured on first use; NULL when capture is not possible, and then never tried again for
 // this context).
@@ -378,6 +389,7 @@ static cudaGraphExec_t step_graph(lbm_ctx* c, const ParamsOf<S>& p, int cur, int
                                   cudaGraphExec_t* slot) {
     if (!LBM_STEP_GRAPHS || c->graphs_failed) return nullptr;
     if (*slot) return *slot;
+    BesideCaptures beside;
     bool ok = c->capture || cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) == cudaSuccess;
     cudaGraph_t g = nullptr;
     if (ok) ok = cudaStreamBeginCapture(c->capture, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
@@ -417,6 +429,7 @@ static int run_part(lbm_ctx* c, const ParamsOf<S>& p, int64_t n) {
     c->last_run = n;
     cudaGraphExec_t g = nullptr;
     if (again) {
+        BesideCaptures beside;
         // the graphs of another length go once nothing is at work that may be a launch of theirs
         if (c->run_len != n && cudaStreamQuery(c->stream) == cudaSuccess) {
             for (cudaGraphExec_t& old : c->run_graph) {
