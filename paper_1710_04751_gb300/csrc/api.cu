@@ -379,15 +379,14 @@ struct BesideCaptures {
 };
 
 // A graph of n steps from buffer `cur`, and of the check of a whole residual interval, in *slot
-// (captured on first use; NULL when capture is not possible, and then never tried again for
-// this context).
+// (captured on first use; NULL when capture is not possible: *failed, and then never tried again).
 #ifndef LBM_STEP_GRAPHS
 #define LBM_STEP_GRAPHS 1
 #endif
 template <typename S>
 static cudaGraphExec_t step_graph(lbm_ctx* c, const ParamsOf<S>& p, int cur, int64_t n, bool check,
-                                  cudaGraphExec_t* slot) {
-    if (!LBM_STEP_GRAPHS || c->graphs_failed) return nullptr;
+                                  cudaGraphExec_t* slot, bool* failed) {
+    if (!LBM_STEP_GRAPHS || *failed) return nullptr;
     if (*slot) return *slot;
     BesideCaptures beside;
     bool ok = c->capture || cudaStreamCreateWithFlags(&c->capture, cudaStreamNonBlocking) == cudaSuccess;
@@ -405,7 +404,7 @@ static cudaGraphExec_t step_graph(lbm_ctx* c, const ParamsOf<S>& p, int cur, int
     if (g) cudaGraphDestroy(g);
     if (!ok) {
         *slot = nullptr;
-        c->graphs_failed = true;
+        *failed = true;
         cudaGetLastError();  // a failed capture leaves no error behind for the next launch
     }
     return *slot;
@@ -419,27 +418,29 @@ static bool capturing(cudaStream_t st) {
     return true;
 }
 
-// Steps up to the next check launched one by one, or as one graph when the run before them was as
-// long: a program that advances a small cavity a few steps at a time spends most of such a call
-// in the launches (10 steps and the fields at 24^3: 81 -> 77 us a call).
-constexpr int64_t kRunMin = 4, kRunMax = 128;
+// Steps up to the next check, launched one by one or as one graph (RunLengths).
 template <typename S>
 static int run_part(lbm_ctx* c, const ParamsOf<S>& p, int64_t n) {
-    const bool again = n >= kRunMin && n <= kRunMax && n == c->last_run && !capturing(c->stream);
-    c->last_run = n;
+    bool replaced;
+    const int slot = c->runs.find(n, &replaced);
     cudaGraphExec_t g = nullptr;
-    if (again) {
+    if (slot >= 0 && !capturing(c->stream)) {
         BesideCaptures beside;
-        // the graphs of another length go once nothing is at work that may be a launch of theirs
-        if (c->run_len != n && cudaStreamQuery(c->stream) == cudaSuccess) {
-            for (cudaGraphExec_t& old : c->run_graph) {
-                if (old) cudaGraphExecDestroy(old);
-                old = nullptr;
+        cudaGraphExec_t* graphs = c->run_graph[slot];
+        if (replaced) {
+            // the graphs of another length go once nothing is at work that may be a launch of theirs
+            if ((graphs[0] || graphs[1]) && cudaStreamQuery(c->stream) != cudaSuccess) {
+                cudaGetLastError();  // not idle: no error of ours
+            } else {
+                for (int b = 0; b < 2; ++b) {
+                    if (graphs[b]) cudaGraphExecDestroy(graphs[b]);
+                    graphs[b] = nullptr;
+                }
+                c->runs.take(slot, n);
+                replaced = false;
             }
-            c->run_len = n;
         }
-        if (c->run_len == n) g = step_graph<S>(c, p, c->cur, n, false, &c->run_graph[c->cur]);
-        else cudaGetLastError();  // not idle: no error of ours
+        if (!replaced) g = step_graph<S>(c, p, c->cur, n, false, &graphs[c->cur], &c->runs.failed);
     }
     if (g) {
         CUDA_OR_FAIL(c, cudaGraphLaunch(g, c->stream));
@@ -462,7 +463,7 @@ static int run_steps(lbm_ctx* c, int64_t n, bool* checked) {
     for (int64_t s = 0; s < n;) {
         // whole residual intervals, aligned with the step count, go as one graph launch
         if (R > 0 && c->steps % R == 0 && n - s >= R) {
-            if (cudaGraphExec_t g = step_graph<S>(c, p, c->cur, R, true, &c->step_graph[c->cur])) {
+            if (cudaGraphExec_t g = step_graph<S>(c, p, c->cur, R, true, &c->step_graph[c->cur], &c->graphs_failed)) {
                 CUDA_OR_FAIL(c, cudaGraphLaunch(g, c->stream));
                 if (R & 1) c->cur ^= 1;
                 c->steps += R;
@@ -922,8 +923,11 @@ void lbm::destroy_context(lbm_ctx* c) {
     {
         DeviceGuard g(c->device);
         wait_stream(c);
-        for (cudaGraphExec_t* g : {&c->step_graph[0], &c->step_graph[1], &c->run_graph[0], &c->run_graph[1]})
-            if (*g) cudaGraphExecDestroy(*g);
+        for (int b = 0; b < 2; ++b) {
+            if (c->step_graph[b]) cudaGraphExecDestroy(c->step_graph[b]);
+            for (auto& graphs : c->run_graph)
+                if (graphs[b]) cudaGraphExecDestroy(graphs[b]);
+        }
         if (c->capture) cudaStreamDestroy(c->capture);
         if (c->own_arena && c->arena) cudaFree(c->arena);
         if (c->host_bits) cudaFreeHost(c->host_bits);

@@ -10,6 +10,7 @@
 
 #include "internal.h"
 #include "lbm.h"
+#include "run_lengths.h"
 
 // NVTX ranges around the C ABI's calls (header-only NVTX 3: no cost without a tool attached;
 // build with -DLBM_NO_NVTX to leave them out).
@@ -55,10 +56,10 @@ struct lbm_ctx {
     // one per starting buffer, captured on a private stream when first needed
     cudaStream_t capture = nullptr;
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
-    // ... and, once a shorter run of steps is asked for twice in a row, run_len steps likewise
-    cudaGraphExec_t run_graph[2] = {nullptr, nullptr};
-    int64_t run_len = 0, last_run = 0;
     bool graphs_failed = false;  // capture not possible here: launch the steps one by one
+    // ... and the runs of steps between checks that `runs` keeps, likewise
+    lbm::RunLengths runs;
+    cudaGraphExec_t run_graph[lbm::RunLengths::kSlots][2] = {};
     // state_fits_l2 of everything a step goes through: this context, the batch or all slabs
     bool in_l2 = false;
     int64_t cell0 = 0;  // global index of cell 0 (slabs of a larger grid), for the initial noise
