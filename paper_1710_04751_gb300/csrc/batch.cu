@@ -752,11 +752,6 @@ extern "C" int lbm_batch_create(int count, const lbm_grid* grids, int lattice,
     if (cudaMemsetAsync(b->d_ntiles, 0, 64, b->stream) != cudaSuccess)
         return bail(bfail(b, LBM_ECUDA, "cudaMemsetAsync failed%s"));
 
-    int64_t copies = 0;  // bytes of one copy of every member's populations: what a step goes through
-    for (int m = 0; m < count; ++m) {
-        const int64_t ncell = (int64_t)grids[m].nx * grids[m].ny * grids[m].nz;
-        copies += (15 + lattice) * ncell * (o.precision == LBM_FP64 ? 8 : 4);
-    }
     for (int m = 0; m < count; ++m) {
         lbm_options mo;
         lbm_default_options(&mo);
@@ -776,7 +771,6 @@ extern "C" int lbm_batch_create(int count, const lbm_grid* grids, int lattice,
         }
         c->owner = b;
         b->members.push_back(c);
-        c->in_l2 = state_fits_l2(copies);
         b->params64.push_back(dev_params<double>(c));
         b->params32.push_back(dev_params<float>(c));
     }

@@ -60,7 +60,8 @@ struct lbm_ctx {
     // ... and the runs of steps between checks that `runs` keeps, likewise
     lbm::RunLengths runs;
     cudaGraphExec_t run_graph[lbm::RunLengths::kSlots][2] = {};
-    // state_fits_l2 of everything a step goes through: this context, the batch or all slabs
+    // state_fits_l2 of what a step goes through: this context or all slabs (a batch's own kernels load
+    // plainly; a member's flag serves its rounds in lbm_init_fields, which step that member alone)
     bool in_l2 = false;
     int64_t cell0 = 0;  // global index of cell 0 (slabs of a larger grid), for the initial noise
 };
