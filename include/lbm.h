@@ -20,11 +20,13 @@
  *    (-,-,-); D3Q7 the first seven.  Stored populations are post-collision: a step is
  *    pull, then collide.
  *  - Every host pointer is caller-owned and only read/written during the call.  Device
- *    memory is library-owned unless the caller passes an arena in lbm_options.
+ *    memory is library-owned unless the caller passes an arena in lbm_options; a context then
+ *    holds no other (CUDA's own, for its graphs of steps, aside).
  *  - Return codes: LBM_OK (0) or a negative LBM_E* code; lbm_last_error(ctx) then holds a
  *    message (lbm_last_error(NULL) for failures without a context).
  *  - A context is not thread-safe.  All work runs on the context's CUDA stream; calls
- *    that return host data synchronise that stream with a bounded wait.
+ *    that return host data synchronise that stream with a bounded wait.  For its first 20 ms
+ *    a wait polls, yielding the processor between polls; then it sleeps between them.
  */
 #ifndef LBM_H
 #define LBM_H

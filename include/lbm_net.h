@@ -12,7 +12,8 @@
  * im2col matrix), FP32 master weights and Adam moments.
  *
  * Errors follow include/lbm.h (LBM_OK or a negative LBM_E* code, the message in
- * lbm_last_error(NULL)).  Device pointers are caller-owned.
+ * lbm_last_error(NULL)), and so do the waits: polling for 20 ms, then sleeping between polls.
+ * Device pointers are caller-owned.
  */
 #ifndef LBM_NET_H
 #define LBM_NET_H

@@ -9,12 +9,16 @@
 // the 128 voxels of the M tile (bx by bz bb = 128, whole x-rows) seen through the tap's
 // shift; the box's out-of-range part -- the zero padding -- arrives as zeros (TMA fill).
 // The box lands in shared memory exactly as the 2D box of an im2col matrix would (rows of
-// BKC channels, 128-byte swizzle for 64 channels, 64-byte swizzle for 32), so the MMA side
-// is the GEMM's: one CTA of 128 threads per 128 x BN tile, warp 0 lane 0 producing into a
-// 4-stage mbarrier ring, warp 1 lane 0 issuing tcgen05.mma into TMEM, all four warps
-// draining the accumulator.  Epilogues: bias + ReLU + BF16 (the forward pass) or FP32 (the
-// input gradient, the convolution of the output gradient with the mirrored weights).
-// Every wait is bounded as in gemm.cu.
+// BKC channels, 128-byte swizzle for 64 channels, 64-byte swizzle for 32).  Three kernels:
+//   conv_bf16_kernel    one tap at a time, the MMA side the GEMM's: one CTA of 128 threads per
+//                       128 x BN tile, warp 0 producing into a 4-stage mbarrier ring, warp 1
+//                       issuing tcgen05.mma into TMEM (an elected lane of each issues), all
+//                       four warps draining the accumulator (grids below 16^3, and 256^3);
+//   conv_x3_kernel      three kx taps side by side in the MMA's N, persistent, 320 threads, up to
+//                       eight stages, epilogue warps of their own (16^3 to 128^3);
+//   conv_wgrad_kernel, conv_wgrad9_kernel   the weight gradient, below.
+// Epilogues: bias + ReLU + BF16 (the forward pass) or FP32 (the input gradient, the convolution
+// of the output gradient with the mirrored weights).  Every wait is bounded as in gemm.cu.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -224,8 +228,8 @@ __device__ __forceinline__ void store32(void* p, const uint32_t (&h)[8]) {
 struct X3Args {
     int N, n, chunks, cin;  // chunks of 32 input channels
     int ntiles, items;      // tiles of BN output channels; (group of MT tiles, channel tile) pairs
-    int by, mt;             // rows per 128-voxel tile, tiles per item
-    int a_bytes;            // one stage's input box: (mt by + 2) n 64 bytes
+    int mt;                 // tiles per item
+    int a_bytes;            // one stage's input box: (mt by + 2) n 64 bytes, by x-rows per 128-voxel tile
     int stage_bytes;        // a_bytes + 9 BN 64
     int stages;
     int mode;
@@ -236,7 +240,7 @@ struct X3Args {
 };
 constexpr int kX3Threads = 320;  // producer, MMA, two sets of four epilogue warps
 
-constexpr int kX3Bias = 304;     // output channels in whole tiles, at most: 6 tiles of 48 and a chunk
+constexpr int kX3Bias = 256;  // output channels in whole tiles, at most: 4 of 64, 5 of 48
 
 // The store of 16 output channels of a row, bias and ReLU applied.  In 32-byte pieces where the
 // rows allow it: a lane's row is a sector of its own, which two 16-byte stores write twice.
@@ -302,10 +306,8 @@ struct X3Item {
 // one: that layer 110 / 92 us, 64^3 32 -> 32 77 / 64, 32^3 64 -> 192 in FP32 80 / 68, 128^3
 // 32 -> 32 234 / 169, 16^3 128 -> 128 (an item per CTA) 35 / 35.  A 96 -> 32 item takes 66 cycles per
 // MMA of 96 columns (48 of math); leaving out either the weights' or the input's loads changes
-// that little, and neither sharing the weights in clusters of two by TMA multicast nor pairs of
-// CTAs with MMAs of M = 256 (-2 to -10% from 64 input channels on, +20% at 32) was worth a second
-// form.  With 32 input channels the epilogue is the longer part: the rows' ends go between warps
-// as quadruples that every lane reads, the bias comes from shared memory, and a lane's channels
+// that little.  With 32 input channels the epilogue is the longer part: the rows' ends go between
+// warps as quadruples that every lane reads, the bias comes from shared memory, and a lane's channels
 // are stored as whole 32-byte sectors.  Before / after those: 64^3 batch 2 32 -> 32 63 / 59 us and
 // in FP32 73 / 68, 128^3 FP32 233 / 203, 32^3 64 -> 192 FP32 67 / 62.
 template <int BN>
@@ -850,7 +852,8 @@ __global__ void __launch_bounds__(128, 1)
     const int gpt = args.cin >> 5;            // channel groups per kz
 
     if (threadIdx.x == 0) {
-        // another CTA timed out: nothing is loaded or stored, but the pair's barriers are kept
+        // another CTA timed out: nothing is stored (the loads and MMAs go on until a wait sees it), and
+        // the pair's barriers are kept
         failed = *static_cast<volatile int*>(args.err) != 0;
         for (int s = 0; s < S; ++s) {
             mbar_init(full + s, 1);
@@ -1124,7 +1127,7 @@ cudaError_t conv_implicit(const __nv_bfloat16* X, int B, int n, int cin, const _
         if (!make_x_map(&tx, X, B, n, cin, 32, n, mt * by1 + 2, 1, 1) ||
             !make_w_map(&tw, W, cout, 27 * cin, ldw, 32, bn))
             return cudaErrorInvalidValue;
-        X3Args a{cout, n, cin / 32, cin, ntiles, (int)(tiles / mt) * ntiles, by1, mt, (mt * by1 + 2) * n * 64, stage,
+        X3Args a{cout, n, cin / 32, cin, ntiles, (int)(tiles / mt) * ntiles, mt, (mt * by1 + 2) * n * 64, stage,
                  std::min(8, kX3Smem / stage), mode, out, bias, cout % 16 == 0 && !((uintptr_t)out & 31), err};
         switch (bn) {
         case 16: return launch_x3<16>(tx, tw, a, st);
