@@ -772,6 +772,8 @@ __global__ void __launch_bounds__(128, 1)
 // wait, three MMAs / two: 64^3 batch 2, 96 -> 32 channels 187 / 163 us, batch 4 535 / 437, 128^3
 // 32 -> 32 370 / 304, 64^3 64 -> 64 118 / 105, 32^3 batch 4, 96 -> 64 125 / 117,
 // batch 2, 192 -> 64 103 / 97.
+// Padding is by zeros of dZ along x and y, of X along z: a non-finite X at an x or y face also reaches
+// the taps that point outward there (times zero), as a non-finite dZ does in the kernel above.
 // The accumulators fill 288 tensor-memory columns: a CTA holds one M tile of 32 output
 // channels and a range of the blocks; where that leaves SMs idle, two CTAs of a cluster share a
 // range and the second adds its sums to the first's through distributed shared memory (a fixed
