@@ -69,18 +69,19 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 }
 
 // The error cell of the kernels' bounded waits.  Kernels get a pointer to `code` and, on a
-// timeout, write the code there (other CTAs poll it) and through `mirror` into page-locked host
-// memory, which the host reads once the kernel is done: no copy after every call.
+// timeout, write the code through `mirror` into page-locked host memory, which the host reads once the
+// kernel is done (no copy after every call), and then there: another stream's CTAs that return
+// because they see it have the mirror written before their own call reads it.
 struct ErrorCell {
     int code, pad;
     int* mirror;
 };
 __device__ __forceinline__ void record_timeout(int* err, int code) {
-    atomicExch(err, code);
     if (int* const m = reinterpret_cast<ErrorCell*>(err)->mirror) {
         *static_cast<volatile int*>(m) = code;
         __threadfence_system();
     }
+    atomicExch(err, code);
 }
 
 // Waits for the phase of `parity` to complete, for at most `limit_ns` nanoseconds, or
